@@ -20,7 +20,7 @@
 //     (planes k-r..k+q), fed by direct loads of the lead planes.
 //   * The b closure planes at each end of s all combine the same cw planes: a block
 //     whose chunk reaches them first streams those planes once per thread and
-//     forms the closure-row sums of every closure plane together, into a scratch
+//     forms the closure-row sums of its closure planes together, into a scratch
 //     buffer that the same thread reads back when it gets to the plane.
 //   * Nodes on a face add the face's penalty (free surface or characteristic SAT).
 // The stage update (2N-storage Runge-Kutta) is fused in the epilogue.  Tiles of one s
@@ -272,8 +272,8 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
   const bool dq_tma = kDqTile && A.mode == kModeStage;
   if (tid == 0) issue_plane(S, 0, tm, i0, j0, kb, member, dq_tma);
   // closure-row sums of the s closure planes this chunk reaches (while the first copy flies)
-  if (active && face_lo && kb < BC) s_closure_sums<T, O, false>(q, met, d, col, scl);
-  if (active && face_hi && ke > d.ns - BC) s_closure_sums<T, O, true>(q, met, d, col, scl);
+  if (active && face_lo && kb < BC) s_closure_sums<T, O, false>(q, met, d, col, scl, kb, ke);
+  if (active && face_hi && ke > d.ns - BC) s_closure_sums<T, O, true>(q, met, d, col, scl, d.ns - ke, d.ns - kb);
 
   auto ld = [&](const T* p, unsigned off) -> T { return active ? __ldg(p + off) : T(0); };
   // streamed once per launch (the RK register): evict-first in the caches
@@ -621,32 +621,40 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 template <int O>
 constexpr int NVQ() { return OpCoef<O>::r + OpCoef<O>::q; }
 
+// Planes of a chunk along s, for `tiles` tiles of nk planes on `slots` resident blocks.  With r =
+// blocks / slots rounds (at least one) of len planes the launch takes about (r + 1) (len + warm)
+// planes' time: the last round is partly full, and a block first spends `warm` planes' time on its
+// queues (measured: two thirds of the queue's length in FP32, where it waits for the loads; a sixth
+// in FP64, where the pipe counts).  Large grids take few long chunks, small ones are cut until the
+// rounds even out.  Per stage, against at most 96 planes and no fewer than 16: 33^3 order 4 FP64 (20
+// blocks on 152 SMs) 481 -> 104 us; 129 x 129 x 97 order 6 FP64 (170 blocks) 2.35 -> 1.37 ms, FP32
+// (255 blocks on 304 slots) 137 -> 125 us; 257 x 241 x 161 curvilinear FP32 629 -> 537 us; 769 x 769
+// x 257 the same (3 chunks; 6 cost 1 %, 16 cost 8 %).
+inline int s_chunk(long long tiles, int nk, int nb, long long slots, double warm) {
+  int best = nk;
+  double best_cost = -1.0;
+  for (int len = nk < 128 ? nk : 128; len >= 1; --len) {
+    const long long nc = (nk + len - 1) / len;
+    if (best_cost >= 0.0 && (len < 3 || nc * nb > 65535)) break;
+    const double rounds = (double)tiles * nc / (double)slots;
+    const double cost = ((rounds > 1.0 ? rounds : 1.0) + 1.0) * (len + warm);
+    if (best_cost < 0.0 || cost < best_cost) {
+      best_cost = cost;
+      best = len;
+    }
+  }
+  return best;
+}
+
 template <typename T, int O, int KIND, int MAP = 0>
 cudaError_t launch_tiled_order(const StageArgs<T>& A, const TmaSet& tm, cudaStream_t st) {
   const int ni = A.d.nq, nj = A.d.nr, nk = A.d.ns - A.slab.ghost_lo - A.slab.ghost_hi;  // computed planes
-  // s chunks: at most 96 planes; when that leaves SM slots idle (few tiles), more chunks
-  // (at least 16 planes each), the count that minimises waves x (chunk + queue warm-up)
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 152;  // GB300
   const long long tiles = (long long)((ni + TX - 1) / TX) * ((nj + TY - 1) / TY) * A.nb;
-  const long long slots = (long long)sms * tiled_min_blocks<T>();
-  int nchunks = (nk + 95) / 96;
-  if (tiles * nchunks < slots) {
-    const int base = nchunks;
-    long long best = -1;
-    for (int nc = base; nc <= base + 8; ++nc) {
-      const int ch = (nk + nc - 1) / nc;
-      if (nc > base && ch < 16) break;
-      const long long waves = (tiles * ((nk + ch - 1) / ch) + slots - 1) / slots;
-      const long long cost = waves * (ch + NVQ<O>());
-      if (best < 0 || cost < best) {
-        best = cost;
-        nchunks = nc;
-      }
-    }
-  }
-  const int chunk = (nk + nchunks - 1) / nchunks;
+  const int chunk = s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(),
+                            sizeof(T) == 4 ? NVQ<O>() * 2.0 / 3.0 : NVQ<O>() / 6.0);
   dim3 grid((ni + TX - 1) / TX, (nj + TY - 1) / TY, ((nk + chunk - 1) / chunk) * A.nb);
   if (grid.z > 65535 || grid.y > 65535) return cudaErrorInvalidConfiguration;
   dim3 block(TX, TY);

@@ -127,10 +127,13 @@ __device__ __forceinline__ void fill_q_rows(QRows<T>& Qr, int tx, int i0, int ow
 //   scratch[(e*b + r)*6 + c]     = sum_p D-[r][p] F_s,c(plane p)
 //   scratch[(e*b + r)*6 + 3 + c] = sum_p D+[r][p] v_c(plane p)
 // over the cw planes p nearest the face (unit spacing; rows of the high end by
-// D+[N-1-i][N-1-j] = -D-[i][j]).  Each scratch row is a plane-sized array.
+// D+[N-1-i][N-1-j] = -D-[i][j]).  Each scratch row is a plane-sized array.  Only the closure rows
+// [row0, row1) are written: the planes of the caller's chunk (another chunk of the same
+// tile forms the others).
 template <typename T, int O, bool HI>
 __device__ __forceinline__ void s_closure_sums(const T* __restrict__ q, const T* __restrict__ met,
-                                               const Dims& d, int col, T* __restrict__ scratch) {
+                                               const Dims& d, int col, T* __restrict__ scratch, int row0 = 0,
+                                               int row1 = OpCoef<O>::b) {
   using C = OpCoef<O>;
   constexpr int BC = C::b;
   const long long fs = d.fs;
@@ -152,6 +155,7 @@ __device__ __forceinline__ void s_closure_sums(const T* __restrict__ q, const T*
     flux(a, sg, F);
 #pragma unroll
     for (int r = 0; r < BC; ++r) {
+      if (sizeof(T) == 8 && (r < row0 || r >= row1)) continue;  // FP64: the pipe's work counts
       const T wm = HI ? -Tab<T, O>::p(r, p) : Tab<T, O>::m(r, p);
       const T wp = HI ? -Tab<T, O>::m(r, p) : Tab<T, O>::p(r, p);
 #pragma unroll
@@ -163,12 +167,14 @@ __device__ __forceinline__ void s_closure_sums(const T* __restrict__ q, const T*
   }
   T* out = scratch + (long long)(HI ? BC : 0) * 6 * d.plane + col;
 #pragma unroll
-  for (int r = 0; r < BC; ++r)
+  for (int r = 0; r < BC; ++r) {
+    if (r < row0 || r >= row1) continue;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       out[(long long)(r * 6 + c) * d.plane] = am[r][c];
       out[(long long)(r * 6 + 3 + c) * d.plane] = ap[r][c];
     }
+  }
 }
 
 }  // namespace sbp
