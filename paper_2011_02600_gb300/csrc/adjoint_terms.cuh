@@ -25,10 +25,9 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
     add_strain(a, u, sb);
     return;
   }
-  const T an = sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
-  const T n[3] = {a[0] / an, a[1] / an, a[2] / an};
-  const T Zp = sqrt((lamJ + T(2) * muJ) / irhoJ);
-  const T Zs = sqrt(muJ / irhoJ);
+  T n[3];
+  const T an = face_normal(a, n);
+  const Impedances<T> Z = impedances(irhoJ, lamJ, muJ);
   const T f = an * inv_h0;
   const T fsg = side == 0 ? f : -f;
   const T cv = T(0.5) * (T(1) - gamma);
@@ -37,12 +36,12 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
   flux(n, ys, w);  // traction of y_sigma on the face
   const T un = yv[0] * n[0] + yv[1] * n[1] + yv[2] * n[2];
   const T wn = w[0] * n[0] + w[1] * n[1] + w[2] * n[2];
-  const T an_ = -f * un + fsg * wn / Zp;
+  const T an_ = -f * un + fsg * wn * Z.iZp;
   T at[3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) at[c] = -f * (yv[c] - un * n[c]) + fsg * (w[c] - wn * n[c]) / Zs;
+  for (int c = 0; c < 3; ++c) at[c] = -f * (yv[c] - un * n[c]) + fsg * (w[c] - wn * n[c]) * Z.iZs;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) vb[c] += cv * (Zp * an_ * n[c] + Zs * at[c]);
+  for (int c = 0; c < 3; ++c) vb[c] += cv * (Z.Zp * an_ * n[c] + Z.Zs * at[c]);
   const T beta[3] = {cT * (an_ * n[0] + at[0]), cT * (an_ * n[1] + at[1]), cT * (an_ * n[2] + at[2])};
   add_strain(n, beta, sb);
 }
@@ -50,10 +49,10 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
 // d/dZp and d/dZs of y . SAT(U) for the general penalty (U = (v, sigma) at the node).
 template <typename T>
 __device__ __forceinline__ void penalty_impedance_derivs(int side, T gamma, T inv_h0, const T v[3], const T s[6],
-                                                         const T yv[3], const T ys[6], const T a[3], T Zp, T Zs,
+                                                         const T yv[3], const T ys[6], const T a[3], T iZp, T iZs,
                                                          T& dZp, T& dZs) {
-  const T an = sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
-  const T n[3] = {a[0] / an, a[1] / an, a[2] / an};
+  T n[3];
+  const T an = face_normal(a, n);
   const T f = an * inv_h0;
   const T fsg = side == 0 ? f : -f;
   const T cv = T(0.5) * (T(1) - gamma);
@@ -71,8 +70,8 @@ __device__ __forceinline__ void penalty_impedance_derivs(int side, T gamma, T in
     vtut += (v[c] - vn * n[c]) * (yv[c] - un * n[c]);
     Ttwt += (Tr[c] - Tn * n[c]) * (w[c] - wn * n[c]);
   }
-  dZp = -f * cv * vn * un - fsg * cT * Tn * wn / (Zp * Zp);
-  dZs = -f * cv * vtut - fsg * cT * Ttwt / (Zs * Zs);
+  dZp = -f * cv * vn * un - fsg * cT * Tn * wn * (iZp * iZp);
+  dZs = -f * cv * vtut - fsg * cT * Ttwt * (iZs * iZs);
 }
 
 // Face terms of L^T at one node: for each face the node lies on, (B H^-1)_xi applied to
@@ -127,8 +126,8 @@ __device__ __forceinline__ void gradient_terms(const T rv[3], const T e[6], cons
   const bool face = pos[0] == 0 || pos[0] == N[0] - 1 || pos[1] == 0 || pos[1] == N[1] - 1 || pos[2] == 0 ||
                     pos[2] == N[2] - 1;
   if (!face) return;
-  const T Zp = sqrt((lamJ + T(2) * muJ) / irhoJ), Zs = sqrt(muJ / irhoJ);
-  const T rT = T(rho), iZp = T(1) / Zp, iZs = T(1) / Zs, i2r = T(0.5) / rT;
+  const Impedances<T> Z = impedances(irhoJ, lamJ, muJ);
+  const T rT = T(rho), i2r = T(0.5) / rT;
   T d_rho = T(0), d_lam = T(0), d_mu = T(0);
 #pragma unroll
   for (int xi = 0; xi < 3; ++xi) {
@@ -138,11 +137,11 @@ __device__ __forceinline__ void gradient_terms(const T rv[3], const T e[6], cons
       if ((side == 0 && !lo) || (side == 1 && !hi)) continue;
       if (bc_kind[2 * xi + side] != 1) continue;
       T dZp, dZs;
-      penalty_impedance_derivs<T>(side, bc_gamma[2 * xi + side], inv_h0[xi], qc, qc + 3, y, y + 3, a[xi], Zp, Zs,
+      penalty_impedance_derivs<T>(side, bc_gamma[2 * xi + side], inv_h0[xi], qc, qc + 3, y, y + 3, a[xi], Z.iZp, Z.iZs,
                                   dZp, dZs);
-      d_rho += (dZp * Zp + dZs * Zs) * i2r;
-      d_lam += dZp * rT * T(0.5) * iZp;
-      d_mu += dZp * rT * iZp + dZs * rT * T(0.5) * iZs;
+      d_rho += (dZp * Z.Zp + dZs * Z.Zs) * i2r;
+      d_lam += dZp * rT * T(0.5) * Z.iZp;
+      d_mu += dZp * rT * Z.iZp + dZs * rT * T(0.5) * Z.iZs;
     }
   }
   g[0] += dt * (double)d_rho;
