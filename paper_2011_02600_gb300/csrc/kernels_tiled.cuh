@@ -116,8 +116,21 @@ __device__ __forceinline__ T dq_at(const Stage<T, 2>& st, int f, int ty, int tx)
   return st.dq[f][ty][tx];
 }
 
-// Fluxes F_q = sigma a_q, F_r = sigma a_r and the strain rows of one axis; MAP 1, 2 skip the
-// products with the components that vanish.
+// a_r for the interior work: on topography maps a_q,x in its place, the constant c of a_r,y = c a_q,x
+// being part of the r spacing's factor there (one product per row instead of one per flux).
+template <typename T>
+__device__ __forceinline__ void ar_raw_at(const Stage<T, 0>& st, int row, int col, T a[3]) {
+  ar_at(st, row, col, T(1), a);
+}
+template <typename T>
+__device__ __forceinline__ void ar_raw_at(const Stage<T, 1>& st, int row, int col, T a[3]) {
+  a[0] = T(0);
+  a[1] = st.jq[row][HX + col];
+  a[2] = T(0);
+}
+
+// Fluxes F_q = sigma a_q, F_r = sigma a_r and the strain rows of one axis (dv: the unscaled
+// derivative, ih: the spacing's factor); MAP 1, 2 skip the products with the components that vanish.
 template <int MAP, typename T>
 __device__ __forceinline__ void flux_q(const T a[3], const T s[6], T F[3]) {
   if constexpr (MAP >= 1) {
@@ -139,23 +152,27 @@ __device__ __forceinline__ void flux_r(const T a[3], const T s[6], T F[3]) {
   }
 }
 template <int MAP, typename T>
-__device__ __forceinline__ void strain_q(const T a[3], const T dv[3], T e[6]) {
+__device__ __forceinline__ void strain_q(const T a[3], T ih, const T dv[3], T e[6]) {
   if constexpr (MAP >= 1) {
-    e[0] += a[0] * dv[0];
-    e[3] += a[0] * dv[1];
-    e[4] += a[0] * dv[2];
+    const T ah = a[0] * ih;
+    e[0] += ah * dv[0];
+    e[3] += ah * dv[1];
+    e[4] += ah * dv[2];
   } else {
-    add_strain(a, dv, e);
+    const T u[3] = {ih * dv[0], ih * dv[1], ih * dv[2]};
+    add_strain(a, u, e);
   }
 }
 template <int MAP, typename T>
-__device__ __forceinline__ void strain_r(const T a[3], const T dv[3], T e[6]) {
+__device__ __forceinline__ void strain_r(const T a[3], T ih, const T dv[3], T e[6]) {
   if constexpr (MAP >= 1) {
-    e[1] += a[1] * dv[1];
-    e[3] += a[1] * dv[0];
-    e[5] += a[1] * dv[2];
+    const T ah = a[1] * ih;
+    e[1] += ah * dv[1];
+    e[3] += ah * dv[0];
+    e[5] += ah * dv[2];
   } else {
-    add_strain(a, dv, e);
+    const T u[3] = {ih * dv[0], ih * dv[1], ih * dv[2]};
+    add_strain(a, u, e);
   }
 }
 
@@ -221,13 +238,22 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 
   const Dims d = A.d;
   const long long fs = d.fs;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int tid = ty * TX + tx;
+  const int tid = threadIdx.y * TX + threadIdx.x;
   int bx, by;
   swizzle_tiles(blockIdx.x + gridDim.x * blockIdx.y, gridDim.x, gridDim.y, bx, by);
   const TileAxis ax = tile_axis(bx, gridDim.x, d.nq, TX, 4);
   const TileAxis ay = tile_axis(by, gridDim.y, d.nr, TY, 1);
   const int i0 = ax.origin, j0 = ay.origin;
+  // One row of the tile per warp.  FP64, where the pipe's work counts: a tile that owns at most half
+  // its width (129 nodes are 32 + 32 + 32 + 4 + 29) takes its nodes in row order over the threads,
+  // so that they fill whole warps; warps without nodes skip the plane's work.  With the products
+  // taken out of the node's work (below, ar_raw_at, strain_q) 129 x 129 x 97 order 6: 1.33 -> 1.19
+  // ms per stage.  In FP32 the same mapping costs 3 to 10 %: addresses that are no longer the
+  // warp's row.
+  const int own_w = ax.own1 - ax.own0, own_h = ay.own1 - ay.own0;
+  const bool packed = sizeof(T) == 8 && own_w <= TX / 2;
+  const int tx = packed ? ax.own0 - i0 + tid % own_w : threadIdx.x;
+  const int ty = packed ? min(ay.own0 - j0 + tid / own_w, TY - 1) : threadIdx.y;
   const int i = i0 + tx, j = j0 + ty;
   // blockIdx.z = chunk + nchunks * member (a batch of independent states).  The computed
   // planes are [klo, khi): the whole local array but a slab's ghost planes.
@@ -237,12 +263,14 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
   const int member = blockIdx.z / nchunks;
   const int kb = klo + (blockIdx.z % nchunks) * chunk;
   const int ke = min(khi, kb + chunk);
-  const bool active = i >= ax.own0 && i < ax.own1 && j >= ay.own0 && j < ay.own1;
+  const bool active = i >= ax.own0 && i < ax.own1 && j >= ay.own0 && j < ay.own1 &&
+                      !(packed && tid >= own_w * own_h);
+  const bool work = __any_sync(0xffffffffu, active);  // the warp owns nodes
   // a tile owning nodes within b of a q face takes its q rows from a per-thread table
   const bool q_edge = ax.own0 < BC || ax.own1 > d.nq - BC;
   const bool r_close = j < BC || j > d.nr - 1 - BC;
   const bool qr_face = i == 0 || i == d.nq - 1 || j == 0 || j == d.nr - 1;
-  const T ihq = A.inv_h[0], ihr = A.inv_h[1], ihs = A.inv_h[2];
+  const T ihq = A.inv_h[0], ihr = MAP >= 1 ? A.inv_h[1] * A.ar_ratio : A.inv_h[1], ihs = A.inv_h[2];
   const long long boff = (long long)member * A.bstride;
   const T* __restrict__ q = A.q + boff;
   T* __restrict__ qout = A.qout + boff;
@@ -265,7 +293,8 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
     mbar_init(&S.bar[1], 1);
     fence_mbar_init();
   }
-  if (q_edge && ty == 0) fill_q_rows<T, O>(S.qrows, tx, i0, ax.own0, ax.own1, d.nq);  // read after the first plane's barrier
+  // read after the first plane's barrier
+  if (q_edge && threadIdx.y == 0) fill_q_rows<T, O>(S.qrows, threadIdx.x, i0, ax.own0, ax.own1, d.nq);
   __syncthreads();
   // the topography-map variant's stages read the RK register from the tile copy
   constexpr bool kDqTile = MAP == 2;
@@ -364,7 +393,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
       const int cl = t % TX;
       const int rr = HX - QF + t / TX;
       T a[3], s[6];
-      ar_at(st, rr, cl, c_r, a);
+      ar_raw_at(st, rr, cl, a);
 #pragma unroll
       for (int c = 0; c < 6; ++c) s[c] = st.state[3 + c][rr][HX + cl];
       T Fv[3];
@@ -384,6 +413,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
       issue_plane(S, sidx ^ 1, tm, i0, j0, k + 1, member, dq_tma);
     }
 
+    if (sizeof(T) == 8 && !work) continue;
     T rv[3] = {T(0), T(0), T(0)};
     T e[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
     T dv[3];
@@ -397,7 +427,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 #pragma unroll
         for (int jj = -R; jj <= Q; ++jj) sv += T(C::alpha(jj)) * st.state[c][HX + ty][HX + tx + jj];
         rv[c] += ihq * sf;
-        dv[c] = ihq * sv;
+        dv[c] = sv;
       }
     } else {
       const int bm = S.qrows.bm[tx], bp = S.qrows.bp[tx];
@@ -414,13 +444,13 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         rv[m] += ihq * sf[m];
-        dv[m] = ihq * sv[m];
+        dv[m] = sv[m];
       }
     }
     {
       T a[3];
       aq_at(st, ty, HX + tx, c_r, a);
-      strain_q<MAP>(a, dv, e);
+      strain_q<MAP>(a, ihq, dv, e);
     }
     // r
     if (!r_close) {
@@ -432,11 +462,11 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 #pragma unroll
         for (int jj = -R; jj <= Q; ++jj) sv += T(C::alpha(jj)) * st.state[c][HX + ty + jj][HX + tx];
         rv[c] += ihr * sf;
-        dv[c] = ihr * sv;
+        dv[c] = sv;
       }
       T a[3];
-      ar_at(st, HX + ty, tx, c_r, a);
-      strain_r<MAP>(a, dv, e);
+      ar_raw_at(st, HX + ty, tx, a);
+      strain_r<MAP>(a, ihr, dv, e);
     } else if (active) {
       // closure row of a node within b of an r face (whole warps: the row is uniform)
       const bool lo = j < BC;
@@ -456,11 +486,11 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         rv[m] += ihr * sf[m];
-        dv[m] = ihr * sv[m];
+        dv[m] = sv[m];
       }
       T a[3];
-      ar_at(st, HX + ty, tx, c_r, a);
-      strain_r<MAP>(a, dv, e);
+      ar_raw_at(st, HX + ty, tx, a);
+      strain_r<MAP>(a, ihr, dv, e);
     }
     // push this plane's lead values (loaded one plane earlier), then fetch the next plane's, so
     // that their latency overlaps the s derivatives, the epilogue and the next plane's q and r
@@ -510,15 +540,23 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
         add_face_penalties(pos, N, a, qc, st.mat[0][ty][tx], st.mat[1][ty][tx], st.mat[2][ty][tx], A.bc_kind,
                            A.bc_gamma, A.inv_h0, rv, e, &A.ifc, member);
       }
+      // FP64 takes dt into the coefficients (6 products fewer per node); in FP32 the rounding of dt c
+      // would bias every step alike
+      constexpr bool kFoldDt = sizeof(T) == 8;
+      const T dt = kFoldDt && A.mode != kModeRhs ? A.dt : T(1);
       T dd[9];
-      apply_P(rv, e, st.mat[0][ty][tx], st.mat[1][ty][tx], st.mat[2][ty][tx], dd);
+      const T m0 = st.mat[0][ty][tx], m1 = st.mat[1][ty][tx], m2 = st.mat[2][ty][tx];
+      if constexpr (kFoldDt)
+        apply_P(rv, e, dt * m0, dt * m1, dt * m2, dd);
+      else
+        apply_P(rv, e, m0, m1, m2, dd);
       if (A.mode == kModeRhs) {
 #pragma unroll
         for (int f = 0; f < 9; ++f) fldw(qout, f)[off] = dd[f];
       } else {
 #pragma unroll
         for (int f = 0; f < 9; ++f) {
-          T dn = A.dt * dd[f];
+          T dn = kFoldDt ? dd[f] : A.dt * dd[f];
           if (A.mode == kModeStage) {
             if constexpr (kDqTile)
               dn += A.rk_a * dq_at(st, f, ty, tx);
