@@ -432,6 +432,16 @@ int sbp_nn_status(uint32_t* bits);
 int sbp_nn_im2col(const void* X, void* Xc, int32_t C, int32_t B, int32_t T, int32_t kw, int32_t pad, void* stream);
 int sbp_nn_col2im(const float* dXc, void* dX, int32_t C, int32_t B, int32_t T, int32_t kw, int32_t pad,
                   void* stream);
+/* im2col of X upsampled by up = 1 or 2 along time (nearest): X [channel][batch *
+ * T / up] -> Xc as above; the upsampled rows are not formed. */
+int sbp_nn_upsample_im2col(const void* X, void* Xc, int32_t C, int32_t B, int32_t T, int32_t up, int32_t kw,
+                           int32_t pad, void* stream);
+/* Backward of a convolution's input through the ReLU before it: col2im of dXc
+ * (FP32, T samples), the pair sums of an upsampling by up = 1 or 2, the mask A > 0;
+ * dZ and A BF16 [channel][batch * T / up].  The sums as col2im, upsample2 and
+ * relu_backward form them. */
+int sbp_nn_conv_relu_backward(const float* dXc, const void* A, void* dZ, int32_t C, int32_t B, int32_t T, int32_t up,
+                              int32_t kw, int32_t pad, void* stream);
 /* Nearest x2 upsampling along time of `rows` rows of length T, BF16 (backward:
  * sum of pairs, FP32 in and out, X = gradient of the upsampled rows). */
 int sbp_nn_upsample2(const void* X, void* Y, int64_t rows, int32_t T, int32_t backward, void* stream);
@@ -447,6 +457,11 @@ int sbp_nn_mse(const float* Y, const float* Tg, void* dY, int64_t n, double* par
  * m, v; also writes the BF16 copy w_bf16 (may be NULL). */
 int sbp_nn_adam(float* w, const float* g, float* m, float* v, void* w_bf16, int64_t n, float lr, float b1, float b2,
                 float eps, int32_t step, void* stream);
+/* The same for `count` tensors (host arrays of device pointers and sizes; w_bf16[i]
+ * may be NULL). */
+int sbp_nn_adam_multi(int32_t count, float* const* w, const float* const* g, float* const* m, float* const* v,
+                      void* const* w_bf16, const int64_t* n, float lr, float b1, float b2, float eps, int32_t step,
+                      void* stream);
 /* Reshape between the last MLP layer's output H [(c T0 + t)][b] and the
  * convolution layout X [c][b T0 + t] (backward: X -> H). */
 int sbp_nn_mlp_to_conv(void* H, void* X, int32_t C, int32_t T0, int32_t B, int32_t backward, void* stream);

@@ -30,7 +30,7 @@ EXPORTED = ("sbp_min_nodes", "sbp_create_grid", "sbp_destroy", "sbp_layout", "sb
             "sbp_set_receivers_xyz", "sbp_record_receivers", "sbp_set_state", "sbp_get_state",
             "sbp_nn_set_gemm_path", "sbp_nn_status", "sbp_set_slab", "sbp_interface_trace", "sbp_set_interface",
             "sbp_probe_fp64_rate", "sbp_set_map_path", "sbp_map_path", "sbp_adjoint_step",
-            "sbp_nn_fourier_features")
+            "sbp_nn_fourier_features", "sbp_nn_upsample_im2col", "sbp_nn_conv_relu_backward", "sbp_nn_adam_multi")
 
 
 class SbpError(RuntimeError):
@@ -97,6 +97,10 @@ def lib(path=None):
         "sbp_set_batch": [P, i32],
         "sbp_nn_gemm": [i32, i32, i32, P, i64, i32, P, i64, i32, P, i64, i32, P, i32, ctypes.c_float, P],
         "sbp_nn_im2col": [P, P, i32, i32, i32, i32, i32, P],
+        "sbp_nn_upsample_im2col": [P, P, i32, i32, i32, i32, i32, i32, P],
+        "sbp_nn_conv_relu_backward": [P, P, P, i32, i32, i32, i32, i32, i32, P],
+        "sbp_nn_adam_multi": [i32, P, P, P, P, P, P, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float,
+                              i32, P],
         "sbp_nn_col2im": [P, P, i32, i32, i32, i32, i32, P],
         "sbp_nn_upsample2": [P, P, i64, i32, i32, P],
         "sbp_nn_relu_backward": [P, P, P, i64, P],
@@ -379,6 +383,22 @@ def sbp_nn_status():
 
 def sbp_nn_im2col(X, Xc, C, B, T, kw, pad, stream):
     _check(lib().sbp_nn_im2col(_ptr(X), _ptr(Xc), C, B, T, kw, pad, stream))
+
+
+def sbp_nn_upsample_im2col(X, Xc, C, B, T, up, kw, pad, stream):
+    _check(lib().sbp_nn_upsample_im2col(_ptr(X), _ptr(Xc), C, B, T, up, kw, pad, stream))
+
+
+def sbp_nn_conv_relu_backward(dXc, A, dZ, C, B, T, up, kw, pad, stream):
+    _check(lib().sbp_nn_conv_relu_backward(_ptr(dXc), _ptr(A), _ptr(dZ), C, B, T, up, kw, pad, stream))
+
+
+def sbp_nn_adam_multi(tensors, lr, b1, b2, eps, step, stream):
+    """tensors: (w, g, m, v, w_bf16 or None) per tensor."""
+    k = len(tensors)
+    cols = [(P * k)(*(None if t[i] is None else t[i].data_ptr() for t in tensors)) for i in range(5)]
+    n = (ctypes.c_int64 * k)(*(t[0].numel() for t in tensors))
+    _check(lib().sbp_nn_adam_multi(k, *cols, n, lr, b1, b2, eps, step, stream))
 
 
 def sbp_nn_col2im(dXc, dX, C, B, T, kw, pad, stream):

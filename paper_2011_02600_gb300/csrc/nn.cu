@@ -317,13 +317,62 @@ __global__ void __launch_bounds__(256) gemm_bf16_pipe_kernel(int M, int N, int K
       }
 }
 
-// im2col of a 1D convolution (kernel width kw, zero padding pad): X [C][B*T] ->
-// Xc [(c*kw + k)][b*T + t] = X[c][b*T + t + k - pad] (zero outside 0..T-1).
+// Eight BF16 values of a row, loaded and stored as 16 bytes.
+struct alignas(16) Bf8 {
+  __nv_bfloat16 v[8];
+};
+
+// im2col of a 1D convolution (kernel width kw, zero padding pad) on X upsampled by `up` along time
+// (nearest): X [C][B*T/up] -> Xc [(c*kw + k)][b*T + t] = X[c][b*T/up + (t + k - pad)/up] (zero where
+// t + k - pad lies outside 0..T-1).  Element by element, for any sizes.
 __global__ void im2col_kernel(const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Xc, int C, int B,
-                              int T, int kw, int pad) {
+                              int T, int up, int kw, int pad) {
   const long long n = (long long)C * kw * B * T;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
-    im2col_at(X, Xc, B, T, kw, pad, e);
+    upsample_im2col_at(X, Xc, B, T, up, kw, pad, e);
+  }
+}
+
+// The same for kw = 5, pad = 2 and T a multiple of 8: a thread takes eight columns of one channel (of
+// one sample, as 8 divides T), reads their window of 12 values once and writes eight columns of the
+// five rows, 16 bytes each.  Bound by the writes (5 times the input; 640 x 32768, 42 MB, in 8.5 us);
+// element by element it was bound by index divisions and 2-byte stores.  UP = 2 reads the row before
+// its upsampling, which is then not formed.  The six calls of the full-size network's forward pass
+// (batch 32): 252 us, and 30 us of upsampling, -> 34 us.
+template <int UP>
+__global__ void __launch_bounds__(256) im2col5_kernel(const __nv_bfloat16* __restrict__ X,
+                                                      __nv_bfloat16* __restrict__ Xc, int N, int T) {
+  const int n = 8 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (n >= N) return;
+  const int c = blockIdx.y;
+  const int t = n % T;  // the sample's first of the eight columns
+  const __nv_bfloat16* x = X + (size_t)c * (N / UP) + n / UP;
+  const __nv_bfloat16 zero = __float2bfloat16(0.f);
+  __nv_bfloat16 w[12];  // columns t - 2 .. t + 9 of the (upsampled) row
+  if (UP == 1) {
+    const Bf8 m = *reinterpret_cast<const Bf8*>(x);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[2 + e] = m.v[e];
+    w[0] = t > 0 ? x[-2] : zero;
+    w[1] = t > 0 ? x[-1] : zero;
+    w[10] = t + 8 < T ? x[8] : zero;
+    w[11] = t + 8 < T ? x[9] : zero;
+  } else {
+    struct alignas(8) Bf4 {
+      __nv_bfloat16 v[4];
+    };
+    const Bf4 m = *reinterpret_cast<const Bf4*>(x);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) w[2 + e] = m.v[e / 2];
+    w[0] = w[1] = t > 0 ? x[-1] : zero;
+    w[10] = w[11] = t + 8 < T ? x[4] : zero;
+  }
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    Bf8 o;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) o.v[e] = w[e + k];
+    *reinterpret_cast<Bf8*>(Xc + (size_t)(5 * c + k) * N + n) = o;
   }
 }
 
@@ -333,6 +382,40 @@ __global__ void col2im_kernel(const float* __restrict__ dXc, float* __restrict__
   const long long n = (long long)C * B * T;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     col2im_at(dXc, dX, B, T, kw, pad, e);
+  }
+}
+
+// From the gradient of a convolution's columns to that of the layer before it: col2im, the pair sums
+// of the x2 upsampling (UP = 2) and the ReLU mask, dZ[c][n] = (A > 0) sum_u col2im(dXc)[UP n + u] in
+// BF16, one pass over the columns in place of three kernels and two FP32 arrays (the six of the
+// full-size network's backward pass, batch 32: 197 -> 85 us; bound by the columns, 84 MB for 32768 of
+// 128 channels).  N = B * T / UP columns of A, Ta = T / UP per sample; a thread
+// takes one.
+template <int UP, int KW>
+__global__ void __launch_bounds__(256) conv_relu_bwd_kernel(const float* __restrict__ dXc,
+                                                            const __nv_bfloat16* __restrict__ A,
+                                                            __nv_bfloat16* __restrict__ dZ, int C, long long N, int Ta,
+                                                            int kw_, int pad) {
+  const long long n = (long long)blockIdx.x * 256 + threadIdx.x;
+  if (n >= N) return;
+  const int kw = KW ? KW : kw_;
+  const int t = N < (1LL << 31) ? (int)n % Ta : (int)(n % Ta), T = UP * Ta;
+  const size_t NT = (size_t)N * UP;
+  for (int c = blockIdx.y; c < C; c += gridDim.y) {
+    const float* x = dXc + (size_t)c * kw * NT + (size_t)UP * (n - t);
+    float du[UP];
+#pragma unroll
+    for (int u = 0; u < UP; ++u) {
+      du[u] = 0.f;
+#pragma unroll
+      for (int k = 0; k < (KW ? KW : kw); ++k) {
+        const int tt = UP * t + u - k + pad;
+        if (tt >= 0 && tt < T) du[u] += x[k * NT + tt];
+      }
+    }
+    const float s = UP == 2 ? du[0] + du[UP - 1] : du[0];
+    const size_t e = (size_t)c * N + n;
+    dZ[e] = __float2bfloat16(__bfloat162float(A[e]) > 0.f ? s : 0.f);
   }
 }
 
@@ -363,19 +446,40 @@ __global__ void relu_bwd_kernel(const float* __restrict__ dA, const __nv_bfloat1
     dZ[e] = __float2bfloat16(__bfloat162float(A[e]) > 0.f ? dA[e] : 0.f);
 }
 
-// db[m] = sum_n dZ[m][n]  (one block per row, fixed order)
-__global__ void bias_grad_kernel(const __nv_bfloat16* __restrict__ dZ, float* __restrict__ db, int M, long long N) {
-  __shared__ float red[256];
-  const int m = blockIdx.x;
+// db[m] = sum_n dZ[m][n], fixed order: TPR threads per row (a warp for short rows, else a block), a
+// thread's values 8 at a time where `wide` (rows 16-byte aligned).  1152 x 32768 (75 MB): 21 -> 14 us;
+// 4096 x 32: 7.2 -> 3.0 us (a block per row had 32 of its 256 threads at work).
+template <int TPR>
+__global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __restrict__ dZ, float* __restrict__ db,
+                                                        int M, long long N, int wide) {
+  __shared__ float red[8];
+  const int m = blockIdx.x * (256 / TPR) + threadIdx.x / TPR, lane = threadIdx.x % TPR;
+  if (TPR < 256 && m >= M) return;  // whole warps
+  const __nv_bfloat16* row = dZ + (size_t)m * N;
   float s = 0.f;
-  for (long long n = threadIdx.x; n < N; n += blockDim.x) s += __bfloat162float(dZ[(long long)m * N + n]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  if (wide) {
+    for (long long n = 8 * lane; n < N; n += 8 * TPR) {
+      const Bf8 x = *reinterpret_cast<const Bf8*>(row + n);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) s += __bfloat162float(x.v[e]);
+    }
+  } else {
+    for (long long n = lane; n < N; n += TPR) s += __bfloat162float(row[n]);
   }
-  if (threadIdx.x == 0) db[m] = red[0];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (TPR == 32) {
+    if (lane == 0) db[m] = s;
+    return;
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float v = 0.f;
+#pragma unroll
+    for (int w = 0; w < TPR / 32; ++w) v += red[w];
+    db[m] = v;
+  }
 }
 
 // mean squared error over n values: per-block FP64 partial sums of (y - t)^2 and dY = 2 (y - t) / n (BF16)
@@ -403,6 +507,42 @@ __global__ void adam_kernel(float* __restrict__ w, const float* __restrict__ g, 
                             float* __restrict__ v, __nv_bfloat16* __restrict__ wb, long long n, float lr, float b1,
                             float b2, float eps, float c1, float c2) {
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
+    const float gi = g[e];
+    const float mi = b1 * m[e] + (1.f - b1) * gi;
+    const float vi = b2 * v[e] + (1.f - b2) * gi * gi;
+    m[e] = mi;
+    v[e] = vi;
+    const float wi = w[e] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[e] = wi;
+    if (wb) wb[e] = __float2bfloat16(wi);
+  }
+}
+
+// Adam over several tensors in one launch (a network's weights and biases: 18 launches, most of a few
+// blocks, 86 -> 27 us for 3.5 M weights): a block takes kAdamChunk values of one tensor.
+constexpr int kAdamTensors = 32, kAdamChunk = 2048;
+struct AdamTensors {
+  float* w[kAdamTensors];
+  const float* g[kAdamTensors];
+  float* m[kAdamTensors];
+  float* v[kAdamTensors];
+  __nv_bfloat16* wb[kAdamTensors];
+  long long n[kAdamTensors];
+  int first[kAdamTensors + 1];  // first block of each tensor
+};
+__global__ void __launch_bounds__(256) adam_multi_kernel(const __grid_constant__ AdamTensors A, int count, float lr,
+                                                         float b1, float b2, float eps, float c1, float c2) {
+  int i = 0;
+  while (i + 1 < count && (int)blockIdx.x >= A.first[i + 1]) ++i;
+  const long long e0 = (long long)((int)blockIdx.x - A.first[i]) * kAdamChunk;
+  const long long e1 = e0 + kAdamChunk < A.n[i] ? e0 + kAdamChunk : A.n[i];
+  float* w = A.w[i];
+  const float* g = A.g[i];
+  float* m = A.m[i];
+  float* v = A.v[i];
+  __nv_bfloat16* wb = A.wb[i];
+#pragma unroll 4
+  for (long long e = e0 + threadIdx.x; e < e1; e += 256) {
     const float gi = g[e];
     const float mi = b1 * m[e] + (1.f - b1) * gi;
     const float vi = b2 * v[e] + (1.f - b2) * gi * gi;
@@ -445,6 +585,48 @@ __global__ void moment_combine_bwd_kernel(const __nv_bfloat16* __restrict__ dy, 
   const long long n = 6LL * n_out * B * T;
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
     moment_combine_bwd_at(dy, m, dG, n_out, B, T, e);
+  }
+}
+
+// The same, eight columns of one sample per thread (T a multiple of 8, 16-byte aligned rows): bound
+// by the trace sets (6 times the traces).  192 traces x 32768 columns: forward (75 + 25 MB) 31 -> 16
+// us, backward (13 + 75 MB) 145 -> 13 us.
+__global__ void __launch_bounds__(256) moment_combine8_kernel(const __nv_bfloat16* __restrict__ G,
+                                                              const float* __restrict__ m, float* __restrict__ y,
+                                                              int n_out, int B, int N, int T) {
+  const int n = 8 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (n >= N) return;
+  const int o = blockIdx.y, b = n / T;
+  float s[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) s[e] = 0.f;
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const Bf8 g = *reinterpret_cast<const Bf8*>(G + ((size_t)c * n_out + o) * N + n);
+    const float mc = m[c * B + b];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) s[e] += mc * __bfloat162float(g.v[e]);
+  }
+  float4* out = reinterpret_cast<float4*>(y + (size_t)o * N + n);
+  out[0] = make_float4(s[0], s[1], s[2], s[3]);
+  out[1] = make_float4(s[4], s[5], s[6], s[7]);
+}
+
+__global__ void __launch_bounds__(256) moment_combine8_bwd_kernel(const __nv_bfloat16* __restrict__ dy,
+                                                                  const float* __restrict__ m,
+                                                                  __nv_bfloat16* __restrict__ dG, int n_out, int B,
+                                                                  int N, int T) {
+  const int n = 8 * (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (n >= N) return;
+  const int o = blockIdx.y, b = n / T;
+  const Bf8 d = *reinterpret_cast<const Bf8*>(dy + (size_t)o * N + n);
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    const float mc = m[c * B + b];
+    Bf8 g;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) g.v[e] = __float2bfloat16(mc * __bfloat162float(d.v[e]));
+    *reinterpret_cast<Bf8*>(dG + ((size_t)c * n_out + o) * N + n) = g;
   }
 }
 
@@ -493,6 +675,11 @@ int nn_bad(const char* msg) {
 int g_gemm_path = 0;
 
 // SM count of the current device (152 on GB300, also the value taken if the query fails).
+bool aligned16(const void* p) { return (uintptr_t)p % 16 == 0; }
+// Rows of B * T columns that a thread can take eight of at a time: one sample's, 16-byte aligned, and
+// few enough for 32-bit indices and a grid row each.
+bool by_eight(long long B, long long T, long long rows) { return T % 8 == 0 && B * T < (1LL << 31) - 2048 && rows <= 65535; }
+
 int device_sms() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -586,11 +773,50 @@ int sbp_nn_status(uint32_t* bits) {
   return SBP_OK;
 }
 
-int sbp_nn_im2col(const void* X, void* Xc, int32_t C, int32_t B, int32_t T, int32_t kw, int32_t pad, void* stream) {
-  if (!X || !Xc || C <= 0 || B <= 0 || T <= 0 || kw <= 0 || pad < 0) return nn_bad("bad im2col arguments");
+int sbp_nn_upsample_im2col(const void* X, void* Xc, int32_t C, int32_t B, int32_t T, int32_t up, int32_t kw,
+                           int32_t pad, void* stream) {
+  if (!X || !Xc || C <= 0 || B <= 0 || T <= 0 || kw <= 0 || pad < 0 || up < 1 || up > 2 || T % up)
+    return nn_bad("bad im2col arguments");
+  const cudaStream_t st = (cudaStream_t)stream;
+  const __nv_bfloat16* x = (const __nv_bfloat16*)X;
+  __nv_bfloat16* xc = (__nv_bfloat16*)Xc;
+  if (kw == 5 && pad == 2 && by_eight(B, T, C) && (uintptr_t)X % (16 / up) == 0 && aligned16(Xc)) {
+    const int N = B * T;
+    const dim3 grid((unsigned)((N / 8 + 255) / 256), (unsigned)C);
+    if (up == 1)
+      im2col5_kernel<1><<<grid, 256, 0, st>>>(x, xc, N, T);
+    else
+      im2col5_kernel<2><<<grid, 256, 0, st>>>(x, xc, N, T);
+    return nn_status(cudaGetLastError());
+  }
   const long long n = (long long)C * kw * B * T;
-  im2col_kernel<<<grid_for(n), 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)X, (__nv_bfloat16*)Xc, C, B, T,
-                                                                kw, pad);
+  im2col_kernel<<<grid_for(n), 256, 0, st>>>(x, xc, C, B, T, up, kw, pad);
+  return nn_status(cudaGetLastError());
+}
+
+int sbp_nn_im2col(const void* X, void* Xc, int32_t C, int32_t B, int32_t T, int32_t kw, int32_t pad, void* stream) {
+  return sbp_nn_upsample_im2col(X, Xc, C, B, T, 1, kw, pad, stream);
+}
+
+int sbp_nn_conv_relu_backward(const float* dXc, const void* A, void* dZ, int32_t C, int32_t B, int32_t T, int32_t up,
+                              int32_t kw, int32_t pad, void* stream) {
+  if (!dXc || !A || !dZ || C <= 0 || B <= 0 || T <= 0 || kw <= 0 || pad < 0 || up < 1 || up > 2 || T % up)
+    return nn_bad("bad conv_relu_backward arguments");
+  const long long N = (long long)B * (T / up);
+  if (N > (1LL << 38)) return nn_bad("too many columns");
+  const cudaStream_t st = (cudaStream_t)stream;
+  const dim3 grid((unsigned)((N + 255) / 256), (unsigned)std::min(C, 65535));
+  const __nv_bfloat16* a = (const __nv_bfloat16*)A;
+  __nv_bfloat16* dz = (__nv_bfloat16*)dZ;
+  const int Ta = T / up;
+  if (kw == 5 && up == 1)
+    conv_relu_bwd_kernel<1, 5><<<grid, 256, 0, st>>>(dXc, a, dz, C, N, Ta, kw, pad);
+  else if (kw == 5)
+    conv_relu_bwd_kernel<2, 5><<<grid, 256, 0, st>>>(dXc, a, dz, C, N, Ta, kw, pad);
+  else if (up == 1)
+    conv_relu_bwd_kernel<1, 0><<<grid, 256, 0, st>>>(dXc, a, dz, C, N, Ta, kw, pad);
+  else
+    conv_relu_bwd_kernel<2, 0><<<grid, 256, 0, st>>>(dXc, a, dz, C, N, Ta, kw, pad);
   return nn_status(cudaGetLastError());
 }
 
@@ -620,7 +846,12 @@ int sbp_nn_relu_backward(const float* dA, const void* A, void* dZ, int64_t n, vo
 
 int sbp_nn_bias_grad(const void* dZ, float* db, int32_t M, int64_t N, void* stream) {
   if (!dZ || !db || M <= 0 || N <= 0) return nn_bad("bad bias_grad arguments");
-  bias_grad_kernel<<<M, 256, 0, (cudaStream_t)stream>>>((const __nv_bfloat16*)dZ, db, M, N);
+  const cudaStream_t st = (cudaStream_t)stream;
+  const int wide = N % 8 == 0 && aligned16(dZ);
+  if (N <= 2048)
+    bias_grad_kernel<32><<<(M + 7) / 8, 256, 0, st>>>((const __nv_bfloat16*)dZ, db, M, N, wide);
+  else
+    bias_grad_kernel<256><<<M, 256, 0, st>>>((const __nv_bfloat16*)dZ, db, M, N, wide);
   return nn_status(cudaGetLastError());
 }
 
@@ -640,6 +871,35 @@ int sbp_nn_adam(float* w, const float* g, float* m, float* v, void* w_bf16, int6
   return nn_status(cudaGetLastError());
 }
 
+int sbp_nn_adam_multi(int32_t count, float* const* w, const float* const* g, float* const* m, float* const* v,
+                      void* const* w_bf16, const int64_t* n, float lr, float b1, float b2, float eps, int32_t step,
+                      void* stream) {
+  if (count <= 0 || !w || !g || !m || !v || !w_bf16 || !n || step < 1) return nn_bad("bad adam arguments");
+  for (int i = 0; i < count; ++i)
+    if (!w[i] || !g[i] || !m[i] || !v[i] || n[i] <= 0) return nn_bad("bad adam arguments");
+  const float c1 = 1.f - powf(b1, (float)step), c2 = 1.f - powf(b2, (float)step);
+  for (int i0 = 0; i0 < count; i0 += kAdamTensors) {
+    AdamTensors A{};
+    const int k = count - i0 < kAdamTensors ? count - i0 : kAdamTensors;
+    long long blocks = 0;
+    for (int i = 0; i < k; ++i) {
+      A.w[i] = w[i0 + i];
+      A.g[i] = g[i0 + i];
+      A.m[i] = m[i0 + i];
+      A.v[i] = v[i0 + i];
+      A.wb[i] = (__nv_bfloat16*)w_bf16[i0 + i];
+      A.n[i] = n[i0 + i];
+      A.first[i] = (int)blocks;
+      blocks += (n[i0 + i] + kAdamChunk - 1) / kAdamChunk;
+      if (blocks > (1LL << 30)) return nn_bad("too many weights");
+    }
+    A.first[k] = (int)blocks;
+    adam_multi_kernel<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(A, k, lr, b1, b2, eps, c1, c2);
+    if (int rc = nn_status(cudaGetLastError())) return rc;
+  }
+  return SBP_OK;
+}
+
 int sbp_nn_mlp_to_conv(void* H, void* X, int32_t C, int32_t T0, int32_t B, int32_t backward, void* stream) {
   if (!H || !X || C <= 0 || T0 <= 0 || B <= 0) return nn_bad("bad reshape arguments");
   mlp_to_conv_kernel<<<grid_for((long long)C * T0 * B), 256, 0, (cudaStream_t)stream>>>(
@@ -650,14 +910,25 @@ int sbp_nn_mlp_to_conv(void* H, void* X, int32_t C, int32_t T0, int32_t B, int32
 int sbp_nn_moment_combine(const void* G, const float* m, float* y, const void* dy, void* dG, int32_t n_out,
                           int32_t B, int32_t T, int32_t backward, void* stream) {
   if (!m || n_out <= 0 || B <= 0 || T <= 0) return nn_bad("bad moment_combine arguments");
+  const cudaStream_t st = (cudaStream_t)stream;
+  const bool eight = by_eight(B, T, n_out);
+  const int N = eight ? B * T : 0;
+  const dim3 grid8((unsigned)((N / 8 + 255) / 256), (unsigned)n_out);
   if (backward) {
     if (!dy || !dG) return nn_bad("moment_combine backward needs dy and dG");
-    moment_combine_bwd_kernel<<<grid_for(6LL * n_out * B * T), 256, 0, (cudaStream_t)stream>>>(
-        (const __nv_bfloat16*)dy, m, (__nv_bfloat16*)dG, n_out, B, T);
+    if (eight && aligned16(dy) && aligned16(dG))
+      moment_combine8_bwd_kernel<<<grid8, 256, 0, st>>>((const __nv_bfloat16*)dy, m, (__nv_bfloat16*)dG, n_out, B, N,
+                                                        T);
+    else
+      moment_combine_bwd_kernel<<<grid_for(6LL * n_out * B * T), 256, 0, st>>>((const __nv_bfloat16*)dy, m,
+                                                                               (__nv_bfloat16*)dG, n_out, B, T);
   } else {
     if (!G || !y) return nn_bad("moment_combine needs G and y");
-    moment_combine_kernel<<<grid_for((long long)n_out * B * T), 256, 0, (cudaStream_t)stream>>>(
-        (const __nv_bfloat16*)G, m, y, n_out, B, T);
+    if (eight && aligned16(G) && aligned16(y))
+      moment_combine8_kernel<<<grid8, 256, 0, st>>>((const __nv_bfloat16*)G, m, y, n_out, B, N, T);
+    else
+      moment_combine_kernel<<<grid_for((long long)n_out * B * T), 256, 0, st>>>((const __nv_bfloat16*)G, m, y, n_out,
+                                                                                B, T);
   }
   return nn_status(cudaGetLastError());
 }

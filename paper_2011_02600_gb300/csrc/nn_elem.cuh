@@ -22,6 +22,18 @@ __device__ __forceinline__ void im2col_at(const __nv_bfloat16* __restrict__ X, _
   Xc[e] = (ts >= 0 && ts < T) ? X[(long long)c * B * T + (long long)b * T + ts] : __float2bfloat16(0.f);
 }
 
+// The same on X upsampled by `up` along time (nearest; X [C][B*T/up])
+__device__ __forceinline__ void upsample_im2col_at(const __nv_bfloat16* __restrict__ X, __nv_bfloat16* __restrict__ Xc,
+                                                   int B, int T, int up, int kw, int pad, long long e) {
+  if (up == 1) return im2col_at(X, Xc, B, T, kw, pad, e);
+  const long long col = e % ((long long)B * T);
+  const long long row = e / ((long long)B * T);
+  const int c = (int)(row / kw), k = (int)(row % kw);
+  const int b = (int)(col / T), t = (int)(col % T);
+  const int ts = t + k - pad, Tx = T / up;
+  Xc[e] = (ts >= 0 && ts < T) ? X[((long long)c * B + b) * Tx + ts / up] : __float2bfloat16(0.f);
+}
+
 // dX[c][b*T + t] = sum_k dXc[(c*kw + k)][b*T + t - k + pad]  (FP32)
 __device__ __forceinline__ void col2im_at(const float* __restrict__ dXc, float* __restrict__ dX, int B, int T, int kw,
                                           int pad, long long e) {

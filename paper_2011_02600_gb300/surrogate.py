@@ -105,11 +105,9 @@ class SurrogateNet:
         cols = []
         T = T0
         for i in range(self.n_up):
-            u = torch.empty(C, B * 2 * T, **bf)
-            L.sbp_nn_upsample2(a, u, C * B, T, 0, _stream())
             T *= 2
             col = torch.empty(C * KW, B * T, **bf)
-            L.sbp_nn_im2col(u, col, C, B, T, KW, PAD, _stream())
+            L.sbp_nn_upsample_im2col(a, col, C, B, T, 2, KW, PAD, _stream())
             a = torch.empty(C, B * T, **bf)
             self._gemm(C, B * T, C * KW, self.wb[f"conv{i}"], C * KW, 0, col, B * T, 0, a, B * T, True,
                        self.b[f"conv{i}"], 1)
@@ -151,25 +149,19 @@ class SurrogateNet:
         L.sbp_nn_bias_grad(dy, self.gb["out"], self.n_last, N, st)
         dcol = torch.empty(C * KW, N, **f32)
         self._gemm(C * KW, N, self.n_last, self.wb["out"], C * KW, 1, dy, N, 0, dcol, N, False)
-        da = torch.empty(C, N, **f32)
-        L.sbp_nn_col2im(dcol, da, C, B, T, KW, PAD, st)
+        # dz: gradient before the ReLU of the layer that made these columns
+        dz = torch.empty(C, N, **bf)
+        L.sbp_nn_conv_relu_backward(dcol, c["acts"][self.n_up], dz, C, B, T, 1, KW, PAD, st)
         for i in reversed(range(self.n_up)):
-            a = c["acts"][i + 1]
-            dz = torch.empty(C, B * T, **bf)
-            L.sbp_nn_relu_backward(da, a, dz, C * B * T, st)
             col = c["cols"][i]
             self._gemm(C, C * KW, B * T, dz, B * T, 0, col, B * T, 1, self.gw[f"conv{i}"], C * KW, False)
             L.sbp_nn_bias_grad(dz, self.gb[f"conv{i}"], C, B * T, st)
             dcol = torch.empty(C * KW, B * T, **f32)
             self._gemm(C * KW, B * T, C, self.wb[f"conv{i}"], C * KW, 1, dz, B * T, 0, dcol, B * T, False)
-            du = torch.empty(C, B * T, **f32)
-            L.sbp_nn_col2im(dcol, du, C, B, T, KW, PAD, st)
+            dz = torch.empty(C, B * (T // 2), **bf)
+            L.sbp_nn_conv_relu_backward(dcol, c["acts"][i], dz, C, B, T, 2, KW, PAD, st)
             T //= 2
-            da = torch.empty(C, B * T, **f32)
-            L.sbp_nn_upsample2(du, da, C * B, T, 1, st)
         # fully connected part (a0 is h3 reshaped)
-        dz = torch.empty(C, B * T0, **bf)
-        L.sbp_nn_relu_backward(da, c["acts"][0], dz, C * B * T0, st)
         dh3 = torch.empty(C * T0, B, **bf)
         L.sbp_nn_mlp_to_conv(dh3, dz, C, T0, B, 1, st)
         self._fc_backward("fc3", dh3, c["h2"], C * T0, H, B)
@@ -191,12 +183,9 @@ class SurrogateNet:
     # ---- optimiser -----------------------------------------------------------
     def adam(self, lr, b1=0.9, b2=0.999, eps=1e-8):
         self.step_count += 1
-        st = _stream()
-        for n in self.names:
-            L.sbp_nn_adam(self.w[n], self.gw[n], self.mw[n], self.vw[n], self.wb[n], self.w[n].numel(), lr, b1, b2,
-                          eps, self.step_count, st)
-            L.sbp_nn_adam(self.b[n], self.gb[n], self.mb[n], self.vb[n], None, self.b[n].numel(), lr, b1, b2, eps,
-                          self.step_count, st)
+        L.sbp_nn_adam_multi([(self.w[n], self.gw[n], self.mw[n], self.vw[n], self.wb[n]) for n in self.names] +
+                            [(self.b[n], self.gb[n], self.mb[n], self.vb[n], None) for n in self.names],
+                            lr, b1, b2, eps, self.step_count, _stream())
 
 
 def mse(y, target, want_grad=True, nblocks=256):
