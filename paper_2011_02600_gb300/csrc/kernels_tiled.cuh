@@ -16,8 +16,9 @@
 //     plane publishes them and frees the stage the next copy will overwrite.
 //   * q and r derivatives read the flux and velocity tiles (interior stencil, or
 //     the closure row of a node within b of the face).  s derivatives use
-//     per-thread register queues of F_s = sigma a_s (planes k-q..k+r) and v
-//     (planes k-r..k+q), fed by direct loads of the lead planes.
+//     per-thread registers, queues of F_s = sigma a_s (planes k-q..k+r) and v
+//     (planes k-r..k+q) or running sums of the derivatives, fed by direct loads
+//     of the lead planes.
 //   * The b closure planes at each end of s all combine the same cw planes: a block
 //     whose chunk reaches them first streams those planes once per thread and
 //     forms the closure-row sums of its closure planes together, into a scratch
@@ -283,11 +284,6 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
   T* wbm = A.wbar ? A.wbar + boff : nullptr;
   const T* yhm = A.yhat ? A.yhat + boff : nullptr;
   const int col = j * d.ldq + i;
-  // node offsets within a field as 32-bit indices from per-field base pointers (a field holds
-  // fewer than 2^31 elements: the host refuses larger grids)
-  auto fld = [&](const T* p, int c) -> const T* { return p + c * fs; };
-  auto fldw = [&](T* p, int c) -> T* { return p + c * fs; };
-
   if (tid == 0) {
     mbar_init(&S.bar[0], 1);
     mbar_init(&S.bar[1], 1);
@@ -304,29 +300,59 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
   if (active && face_lo && kb < BC) s_closure_sums<T, O, false>(q, met, d, col, scl, kb, ke);
   if (active && face_hi && ke > d.ns - BC) s_closure_sums<T, O, true>(q, met, d, col, scl, d.ns - ke, d.ns - kb);
 
-  auto ld = [&](const T* p, unsigned off) -> T { return active ? __ldg(p + off) : T(0); };
-  // streamed once per launch (the RK register): evict-first in the caches
-  auto ld_stream = [&](const T* p, unsigned off) -> T { return active ? __ldcs(p + off) : T(0); };
-  // plane kk of field c of p at this thread's column; zero outside the grid
-  auto ldk = [&](const T* p, int c, int kk) -> T {
-    return active && kk >= 0 && kk < d.ns ? __ldg(fld(p, c) + ((unsigned)kk * (unsigned)d.plane + (unsigned)col))
-                                          : T(0);
+  // Global accesses: a plane of a field (an address all threads share) and the thread's node in it;
+  // a thread without a node of its own reads one of the tile's.
+  const unsigned at = (unsigned)(active ? col : max(ay.own0, 0) * d.ldq + ax.own0);
+  auto plane_of = [&](const T* p, int c, int kk) -> const T* { return p + (c * fs + (long long)kk * d.plane); };
+  auto plane_w = [&](T* p, int c, int kk) -> T* { return p + (c * fs + (long long)kk * d.plane); };
+  // field c of p at plane kk, for the s derivatives (a plane outside the grid, which only closure
+  // planes' unused sums take in, repeats the nearest)
+  auto ldk = [&](const T* p, int c, int kk) -> T { return __ldg(plane_of(p, c, min(max(kk, 0), d.ns - 1)) + at); };
+  // s derivatives, FP32 on topography maps: running sums, one per plane in flight; a new plane's F_s
+  // (or v) is added with its weight to each plane it reaches, and the shift along the march is the
+  // destination register of the multiply-add.  Otherwise a queue of the planes' F_s and v, with 36
+  // moves a plane at order 6: in FP64 it costs no work of that pipe while it fills, and next to the
+  // nine metric fields the sums are slower (257 x 241 x 161: 515 against 558 us a stage).  With the
+  // sums, addresses formed once per plane and fluxes formed a row per warp, 769 x 769 x 257 order 6:
+  // 5.75 -> 5.57 ms a stage.
+  constexpr bool kSums = sizeof(T) == 4 && MAP >= 1;
+  constexpr int NQ = kSums ? NV - 1 : NV;
+  T vq[NQ][3];  // v at planes k-R .. k+Q, or the sums of D+ v at planes k .. k+NV-2
+  T fq[NQ][3];  // F_s at planes k-Q .. k+R, or the sums of D- F_s
+  auto push = [&](T sums[NQ][3], const T x[3], auto coef, T out[3]) {  // coef(m): weight for plane k + m
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      out[c] = sums[0][c] + T(coef(0)) * x[c];
+#pragma unroll
+      for (int m = 0; m < NQ - 1; ++m) sums[m][c] = sums[m + 1][c] + T(coef(m + 1)) * x[c];
+      sums[NQ - 1][c] = T(coef(NQ)) * x[c];
+    }
   };
-  T vq[NV][3];  // v at planes k-R .. k+Q
-  T fq[NV][3];  // F_s at planes k-Q .. k+R
+  auto coef_f = [](int m) { return -C::alpha(m - R); };  // F_s of plane k + R in D- at plane k + m
+  auto coef_v = [](int m) { return C::alpha(Q - m); };   // v of plane k + Q in D+ at plane k + m
+#pragma unroll
+  for (int m = 0; m < NQ; ++m)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) vq[m][c] = fq[m][c] = T(0);
 #pragma unroll
   for (int m = 0; m < NV - 1; ++m) {
+    T v[3], s[6], a[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) vq[m][c] = ldk(q, c, kb - R + m);
-  }
-#pragma unroll
-  for (int m = 0; m < NV - 1; ++m) {
-    T s[6], a[3];
+    for (int c = 0; c < 3; ++c) v[c] = ldk(q, c, kb - R + m);
 #pragma unroll
     for (int c = 0; c < 6; ++c) s[c] = ldk(q, 3 + c, kb - Q + m);
 #pragma unroll
     for (int c = 0; c < 3; ++c) a[c] = ldk(met, 6 + c, kb - Q + m);
-    flux(a, s, fq[m]);
+    if constexpr (kSums) {
+      T F[3], out[3];
+      flux(a, s, F);
+      push(fq, F, coef_f, out);
+      push(vq, v, coef_v, out);
+    } else {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) vq[m][c] = v[c];
+      flux(a, s, fq[m]);
+    }
   }
 
   // lead values (v at k+Q, sigma and a_s at k+R) staged one plane ahead
@@ -344,7 +370,6 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
   for (int it = 0, k = kb; k < ke; ++it, ++k) {
     const int sidx = it & 1;
     const unsigned phase = (it >> 1) & 1;
-    const unsigned off = (unsigned)k * (unsigned)d.plane + (unsigned)col;
     // the epilogue's own inputs at this node, fetched before the tile wait so that their
     // latency overlaps the plane's derivatives: the RK register (forward stage), Ub_{k+1} and
     // Wb_k (L^T pass), Wb_k, rho and J (gradient pass)
@@ -352,20 +377,20 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
     double rj[2];
     if (KIND == 0 && !kDqTile && A.mode == kModeStage) {
 #pragma unroll
-      for (int c = 0; c < 9; ++c) dqi[c] = ld_stream(fld(dqm, c), off);
+      for (int c = 0; c < 9; ++c) dqi[c] = active ? __ldcs(plane_of(dqm, c, k) + at) : T(0);  // streamed once per launch
     }
     if (KIND == 1 && A.mode != kModeRhs) {
 #pragma unroll
       for (int c = 0; c < 9; ++c) {
-        dqi[c] = ub_next ? ld(fld(ub_next, c), off) : T(0);
-        pre[c] = ld(fld(wbm, c), off);
+        dqi[c] = active && ub_next ? __ldg(plane_of(ub_next, c, k) + at) : T(0);
+        pre[c] = active ? __ldg(plane_of(wbm, c, k) + at) : T(0);
       }
     }
     if (KIND == 2) {
 #pragma unroll
-      for (int c = 0; c < 9; ++c) pre[c] = ld(fld(wbm, c), off);
-      rj[0] = active ? __ldg(A.rlmj + off) : 0.0;
-      rj[1] = active ? __ldg(A.rlmj + 3 * fs + off) : 0.0;
+      for (int c = 0; c < 9; ++c) pre[c] = active ? __ldg(plane_of(wbm, c, k) + at) : T(0);
+      rj[0] = __ldg(A.rlmj + (long long)k * d.plane + at);
+      rj[1] = __ldg(A.rlmj + (3 * fs + (long long)k * d.plane) + at);
     }
 
     // Each thread waits for the plane's copy with a bounded wait; the block decides together
@@ -377,9 +402,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
     FluxTiles<T>& F = S.f[sidx];
     // fluxes on the tile and its halo: F_q at columns -QF..TX-1+R, F_r at rows -QF..TY-1+R
     constexpr int QF = flux_halo<O>();
-    for (int t = tid; t < TY * (QF + R + TX); t += TX * TY) {
-      const int row = t / (QF + R + TX);
-      const int cc = HX - QF + t % (QF + R + TX);
+    auto form_q = [&](int row, int cc) {
       T a[3], s[6];
       aq_at(st, row, cc, c_r, a);
 #pragma unroll
@@ -388,6 +411,14 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
       flux_q<MAP>(a, s, Fv);
 #pragma unroll
       for (int c = 0; c < 3; ++c) F.fq[c][row][cc] = Fv[c];
+    };
+    // a row per warp, then the columns past the tile's width by the last warps (the first ones take
+    // the second round of F_r's rows)
+    form_q(tid / TX, HX - QF + tid % TX);
+    constexpr int kMore = QF + R;
+    if (kMore > 0 && tid >= TX * TY - TY * kMore) {
+      const int e = tid - (TX * TY - TY * kMore);
+      form_q(e / (kMore > 0 ? kMore : 1), HX - QF + TX + e % (kMore > 0 ? kMore : 1));
     }
     for (int t = tid; t < TX * (QF + R + TY); t += TX * TY) {
       const int cl = t % TX;
@@ -495,19 +526,32 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
     // push this plane's lead values (loaded one plane earlier), then fetch the next plane's, so
     // that their latency overlaps the s derivatives, the epilogue and the next plane's q and r
     // derivatives
+    T us[3], uv[3];  // D- F_s and D+ v at this plane (FP32)
+    if constexpr (kSums) {
+      T Fl[3];
+      flux(la, ls, Fl);
+      push(fq, Fl, coef_f, us);
+      push(vq, lv, coef_v, uv);
+    } else {
 #pragma unroll
-    for (int c = 0; c < 3; ++c) vq[NV - 1][c] = lv[c];
-    flux(la, ls, fq[NV - 1]);
+      for (int c = 0; c < 3; ++c) vq[NQ - 1][c] = lv[c];
+      flux(la, ls, fq[NQ - 1]);
+    }
     if (k + 1 < ke) load_lead(k + 1);
     // s (closure rows only within b of a face of the whole block)
     if ((k >= BC || !face_lo) && (k <= d.ns - 1 - BC || !face_hi)) {
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         T sf = T(0), sv = T(0);
+        if constexpr (kSums) {
+          sf = us[c];
+          sv = uv[c];
+        } else {
 #pragma unroll
-        for (int jj = -Q; jj <= R; ++jj) sf += T(-C::alpha(-jj)) * fq[Q + jj][c];
+          for (int jj = -Q; jj <= R; ++jj) sf += T(-C::alpha(-jj)) * fq[Q + jj][c];
 #pragma unroll
-        for (int jj = -R; jj <= Q; ++jj) sv += T(C::alpha(jj)) * vq[R + jj][c];
+          for (int jj = -R; jj <= Q; ++jj) sv += T(C::alpha(jj)) * vq[R + jj][c];
+        }
         rv[c] += ihs * sf;
         dv[c] = ihs * sv;
       }
@@ -552,7 +596,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
         apply_P(rv, e, m0, m1, m2, dd);
       if (A.mode == kModeRhs) {
 #pragma unroll
-        for (int f = 0; f < 9; ++f) fldw(qout, f)[off] = dd[f];
+        for (int f = 0; f < 9; ++f) plane_w(qout, f, k)[at] = dd[f];
       } else {
 #pragma unroll
         for (int f = 0; f < 9; ++f) {
@@ -563,8 +607,8 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
             else
               dn += A.rk_a * dqi[f];
           }
-          __stcs(fldw(dqm, f) + off, dn);                    // read again one stage later
-          __stcs(fldw(qout, f) + off, qc[f] + A.rk_b * dn);
+          __stcs(plane_w(dqm, f, k) + at, dn);                    // read again one stage later
+          __stcs(plane_w(qout, f, k) + at, qc[f] + A.rk_b * dn);
         }
       }
     } else if (active) {
@@ -602,12 +646,12 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
         const T m9[9] = {vb[0], vb[1], vb[2], sb[0], sb[1], sb[2], sb[3], sb[4], sb[5]};
         if (A.mode == kModeRhs) {
 #pragma unroll
-          for (int f = 0; f < 9; ++f) fldw(ub_out, f)[off] = m9[f];
+          for (int f = 0; f < 9; ++f) plane_w(ub_out, f, k)[at] = m9[f];
         } else if (!A.yhat_next) {
 #pragma unroll
           for (int f = 0; f < 9; ++f) {
-            fldw(ub_out, f)[off] = dqi[f] + A.dt * m9[f];
-            fldw(wbm, f)[off] = A.rk_a * pre[f];
+            plane_w(ub_out, f, k)[at] = dqi[f] + A.dt * m9[f];
+            plane_w(wbm, f, k)[at] = A.rk_a * pre[f];
           }
         } else {
           // and the prep of stage k - 1, pointwise at this node: Wb_{k-1} = A_k Wb_k + B_{k-1} Ub_k,
@@ -616,9 +660,9 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 #pragma unroll
           for (int f = 0; f < 9; ++f) {
             const T ub = dqi[f] + A.dt * m9[f];
-            fldw(ub_out, f)[off] = ub;
+            plane_w(ub_out, f, k)[at] = ub;
             w[f] = A.rk_a * pre[f] + A.rk_b_next * ub;
-            fldw(wbm, f)[off] = w[f];
+            plane_w(wbm, f, k)[at] = w[f];
           }
           T y[9];
           apply_P(w, w + 3, irhoJ, lamJ, muJ, y);
@@ -626,7 +670,7 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
                        norm_weight_inv_t<T, O>(k, d.ns) * A.inv_h[2];
           T* yn = A.yhat_next + boff;
 #pragma unroll
-          for (int f = 0; f < 9; ++f) fldw(yn, f)[off] = y[f] * ih;
+          for (int f = 0; f < 9; ++f) plane_w(yn, f, k)[at] = y[f] * ih;
         }
       } else {
         // dt Wb_k . d(P~ M U_k)/d(rho, lambda, mu) at the node
@@ -635,23 +679,25 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
           const T H = norm_weight_t<T, O>(i, d.nq) * A.h[0] * norm_weight_t<T, O>(j, d.nr) * A.h[1] *
                       norm_weight_t<T, O>(k, d.ns) * A.h[2];
 #pragma unroll
-          for (int f = 0; f < 9; ++f) y[f] = H * fld(yhm, f)[off];
+          for (int f = 0; f < 9; ++f) y[f] = H * plane_of(yhm, f, k)[at];
         }
         double g[3];
         gradient_terms(rv, e, qc, pre, y, pos, N, a, irhoJ, lamJ, muJ, rj[0], rj[1], A.bc_kind, A.bc_gamma,
                        A.inv_h0, (double)A.dt, g);
         // one writer per node and launch: a reduction that needs no read-back
 #pragma unroll
-        for (int c = 0; c < 3; ++c) atomicAdd(A.grad + c * fs + off, g[c]);
+        for (int c = 0; c < 3; ++c) atomicAdd(A.grad + (c * fs + (long long)k * d.plane) + at, g[c]);
       }
     }
+    if constexpr (!kSums) {
 #pragma unroll
-    for (int m = 0; m < NV - 1; ++m)
+      for (int m = 0; m < NQ - 1; ++m)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        vq[m][c] = vq[m + 1][c];
-        fq[m][c] = fq[m + 1][c];
-      }
+        for (int c = 0; c < 3; ++c) {
+          vq[m][c] = vq[m + 1][c];
+          fq[m][c] = fq[m + 1][c];
+        }
+    }
   }
 }
 
