@@ -705,31 +705,6 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
 template <int O>
 constexpr int NVQ() { return OpCoef<O>::r + OpCoef<O>::q; }
 
-// Planes of a chunk along s, for `tiles` tiles of nk planes on `slots` resident blocks.  With r =
-// blocks / slots rounds (at least one) of len planes the launch takes about (r + 1) (len + warm)
-// planes' time: the last round is partly full, and a block first spends `warm` planes' time on its
-// queues (measured: two thirds of the queue's length in FP32, where it waits for the loads; a sixth
-// in FP64, where the pipe counts).  Large grids take few long chunks, small ones are cut until the
-// rounds even out.  Per stage, against at most 96 planes and no fewer than 16: 33^3 order 4 FP64 (20
-// blocks on 152 SMs) 481 -> 104 us; 129 x 129 x 97 order 6 FP64 (170 blocks) 2.35 -> 1.37 ms, FP32
-// (255 blocks on 304 slots) 137 -> 125 us; 257 x 241 x 161 curvilinear FP32 629 -> 537 us; 769 x 769
-// x 257 the same (3 chunks; 6 cost 1 %, 16 cost 8 %).
-inline int s_chunk(long long tiles, int nk, int nb, long long slots, double warm) {
-  int best = nk;
-  double best_cost = -1.0;
-  for (int len = nk < 128 ? nk : 128; len >= 1; --len) {
-    const long long nc = (nk + len - 1) / len;
-    if (best_cost >= 0.0 && (len < 3 || nc * nb > 65535)) break;
-    const double rounds = (double)tiles * nc / (double)slots;
-    const double cost = ((rounds > 1.0 ? rounds : 1.0) + 1.0) * (len + warm);
-    if (best_cost < 0.0 || cost < best_cost) {
-      best_cost = cost;
-      best = len;
-    }
-  }
-  return best;
-}
-
 template <typename T, int O, int KIND, int MAP = 0>
 cudaError_t launch_tiled_order(const StageArgs<T>& A, const TmaSet& tm, cudaStream_t st) {
   const int ni = A.d.nq, nj = A.d.nr, nk = A.d.ns - A.slab.ghost_lo - A.slab.ghost_hi;  // computed planes
@@ -737,8 +712,9 @@ cudaError_t launch_tiled_order(const StageArgs<T>& A, const TmaSet& tm, cudaStre
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 152;  // GB300
   const long long tiles = (long long)((ni + TX - 1) / TX) * ((nj + TY - 1) / TY) * A.nb;
-  const int chunk = s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(),
-                            sizeof(T) == 4 ? NVQ<O>() * 2.0 / 3.0 : NVQ<O>() / 6.0);
+  const int chunk = sizeof(T) == 4
+                        ? s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(), NVQ<O>() * 0.6, OpCoef<O>::b, 6)
+                        : s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(), NVQ<O>() / 6.0, OpCoef<O>::b, 1);
   dim3 grid((ni + TX - 1) / TX, (nj + TY - 1) / TY, ((nk + chunk - 1) / chunk) * A.nb);
   if (grid.z > 65535 || grid.y > 65535) return cudaErrorInvalidConfiguration;
   dim3 block(TX, TY);

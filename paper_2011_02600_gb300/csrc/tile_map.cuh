@@ -1,6 +1,6 @@
 // Tile geometry of the tiled stage kernel (kernels_tiled.cu): tile size and halo, the node
 // range each tile owns along q and r, the launch order of the tiles, the per-thread rows of D-
-// and D+ along q, and the closure-row sums along s.  Device code of the kernel; without nvcc the same source compiles as
+// and D+ along q, the closure-row sums along s, and the length of the chunks along s.  Device code of the kernel; without nvcc the same source compiles as
 // host C++, so that the index arithmetic can be checked for any grid size on a CPU.
 #pragma once
 
@@ -175,6 +175,35 @@ __device__ __forceinline__ void s_closure_sums(const T* __restrict__ q, const T*
       out[(long long)(r * 6 + 3 + c) * d.plane] = ap[r][c];
     }
   }
+}
+
+// Planes of a chunk along s, for `tiles` tiles of nk planes on `slots` resident blocks: r = blocks /
+// slots rounds (at least one) of len planes and then one more for the last round's rest, each with
+// `warm` planes' time for a block to fill its queues (0.6 of their length in FP32, where it waits
+// for the loads, a sixth in FP64, where the pipe counts).  The last chunk also forms the closure
+// sums at s = 1 (`extra` planes' time), and the one before it does when the last holds fewer than the
+// b closure planes.  Large grids take few long chunks, small ones are cut until the rounds even out.
+// Per stage, against at most 96 planes and no fewer than 16: 33^3 order 4 FP64 (20 blocks on 152 SMs)
+// 481 -> 79 us; 129 x 129 x 97 order 6 FP64 (170 blocks) 2.35 -> 1.18 ms, FP32 (255 blocks on 304
+// slots) 137 -> 112 us; 257 x 241 x 161 curvilinear FP32 629 -> 514 us, other gains of this kernel
+// included; 769 x 769 x 257 takes 3 chunks (6 cost 1 %, 16 cost 8 %).
+inline int s_chunk(long long tiles, int nk, int nb, long long slots, double warm, int b, int extra) {
+  int best = nk;
+  double best_cost = -1.0;
+  for (int len = nk < 128 ? nk : 128; len >= 1; --len) {
+    const long long nc = (nk + len - 1) / len;
+    if (best_cost >= 0.0 && nc * nb > 65535) break;
+    const int rest = (int)(nk - (nc - 1) * len);  // the last chunk's planes
+    const int before = nc > 1 ? len + (rest < b ? extra : 0) : 0;
+    const double rounds = (double)tiles * nc / (double)slots;
+    const double cost = (rounds > 1.0 ? rounds : 1.0) * (len + warm) +
+                        ((before > rest + extra ? before : rest + extra) + warm);
+    if (best_cost < 0.0 || cost < best_cost) {
+      best_cost = cost;
+      best = len;
+    }
+  }
+  return best;
 }
 
 }  // namespace sbp
