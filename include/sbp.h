@@ -344,6 +344,13 @@ int sbp_adjoint_stage(SbpGrid* grid, int32_t stage, double dt, const void* u_sta
  * sbp_adjoint_stage. */
 int sbp_adjoint_step(SbpGrid* grid, double dt, const void* u_stages, void* ubar, void* wbar, void* scratch,
                      const double* rlmj, double* grad, void* stream);
+/* The stage inputs of one step for sbp_adjoint_step: u_stages holds U_0 in its first
+ * group of states (5 groups of 9 B fields, grid layout) and receives U_1 .. U_4 in the
+ * others, at the grid's time (sbp_set_time; the source's stage times).  Uses the
+ * Runge-Kutta register; the bound state, time and step counter stay as they are.
+ * u_stages: 256-byte aligned, not a bound buffer.
+ * Errors: UNSUPPORTED on slab grids and with interface faces. */
+int sbp_stage_inputs(SbpGrid* grid, double dt, void* u_stages, void* stream);
 
 /* Receiver misfit of the B states q (9 B fields): for member b, receiver r and
  * velocity component c, diff = v_c - data[(b n + r) 3 + c] (data: FP64 device,

@@ -30,7 +30,8 @@ EXPORTED = ("sbp_min_nodes", "sbp_create_grid", "sbp_destroy", "sbp_layout", "sb
             "sbp_set_receivers_xyz", "sbp_record_receivers", "sbp_set_state", "sbp_get_state",
             "sbp_nn_set_gemm_path", "sbp_nn_status", "sbp_set_slab", "sbp_interface_trace", "sbp_set_interface",
             "sbp_probe_fp64_rate", "sbp_set_map_path", "sbp_map_path", "sbp_adjoint_step",
-            "sbp_nn_fourier_features", "sbp_nn_upsample_im2col", "sbp_nn_conv_relu_backward", "sbp_nn_adam_multi")
+            "sbp_nn_fourier_features", "sbp_nn_upsample_im2col", "sbp_nn_conv_relu_backward", "sbp_nn_adam_multi",
+            "sbp_stage_inputs")
 
 
 class SbpError(RuntimeError):
@@ -97,6 +98,7 @@ def lib(path=None):
         "sbp_set_batch": [P, i32],
         "sbp_nn_gemm": [i32, i32, i32, P, i64, i32, P, i64, i32, P, i64, i32, P, i32, ctypes.c_float, P],
         "sbp_nn_im2col": [P, P, i32, i32, i32, i32, i32, P],
+        "sbp_stage_inputs": [P, dbl, P, P],
         "sbp_nn_upsample_im2col": [P, P, i32, i32, i32, i32, i32, i32, P],
         "sbp_nn_conv_relu_backward": [P, P, P, i32, i32, i32, i32, i32, i32, P],
         "sbp_nn_adam_multi": [i32, P, P, P, P, P, P, ctypes.c_float, ctypes.c_float, ctypes.c_float, ctypes.c_float,
@@ -316,6 +318,10 @@ def sbp_energy_noalloc(q, mat, nodes, ldq, fs, order, precision, nblocks, stream
 
 def sbp_rhs_adjoint(h, w, out, scratch, stream):
     _check(lib().sbp_rhs_adjoint(h, _ptr(w), _ptr(out), _ptr(scratch), stream))
+
+
+def sbp_stage_inputs(h, dt, u_stages, stream):
+    _check(lib().sbp_stage_inputs(h, dt, _ptr(u_stages), stream))
 
 
 def sbp_adjoint_step(h, dt, u_stages, ubar, wbar, scratch, rlmj, grad, stream):

@@ -124,10 +124,9 @@ class MisfitProblem:
                 states.append(s.qbuf[s.current].clone())
             for n in reversed(range(seg, end)):
                 L.sbp_misfit(s.h, states[n + 1 - seg], self.data[n], self.dt, None, ubar, st)
-                self._load(states[n - seg], n)
-                for k in range(5):
-                    stage_in[k].copy_(s.qbuf[s.current])
-                    L.sbp_rk_stage(s.h, k, self.dt, st)
+                stage_in[0].copy_(states[n - seg])
+                s.set_time(n * self.dt, n)
+                L.sbp_stage_inputs(s.h, self.dt, stages, st)
                 wbar.zero_()
                 if self.fused:
                     L.sbp_adjoint_step(s.h, self.dt, stages, ubar, wbar, scratch, self.rlmj, grad, st)
@@ -135,6 +134,8 @@ class MisfitProblem:
                     for k in reversed(range(5)):
                         L.sbp_adjoint_stage(s.h, k, self.dt, stage_in[k], ubar, wbar, scratch, self.rlmj, grad,
                                             st)
+            if seg == 0:                        # the solver is left after the first step, as by its five stages
+                self._load(states[min(1, end)], 0)
             del states
         return s.view(grad, 3).clone()
 
