@@ -106,12 +106,11 @@ __device__ __forceinline__ void adjoint_face_terms(const int pos[3], const int N
 // r = 1/(rho J), lambda/J, mu/J.  The three contractions are formed in the state's
 // precision and scaled in FP64 by factors that need no division, 1/(rho^2 J) = r (r J) and
 // 1/J = r rho, so that their tiny magnitudes cannot underflow; dt goes into r once (FP64
-// products are what this pass issues slowest: 7 instead of 9 a node, 8 x 129^3 gradient 315.7
-// -> 311.8 ms).  At faces with the
-// characteristic penalty the impedances Z_p = sqrt(rho (lambda + 2 mu)) and
-// Z_s = sqrt(rho mu) add their derivatives, in the state's precision through
-// dZp/drho = Zp/(2 rho), dZp/dlambda = rho/(2 Zp), dZp/dmu = rho/Zp, dZs/drho = Zs/(2 rho),
-// dZs/dmu = rho/(2 Zs).
+// products are what this pass issues slowest: 7 instead of 9 a node took a 16-step gradient of
+// 8 sources on 129 x 129 x 97 nodes from 315.7 to 311.8 ms).  At faces with the characteristic penalty the
+// impedances Z_p = sqrt(rho (lambda + 2 mu)) and Z_s = sqrt(rho mu) add their derivatives, in the
+// state's precision through dZp/drho = Zp/(2 rho), dZp/dlambda = rho/(2 Zp), dZp/dmu = rho/Zp,
+// dZs/drho = Zs/(2 rho), dZs/dmu = rho/(2 Zs).
 template <typename T>
 __device__ __forceinline__ void gradient_terms(const T rv[3], const T e[6], const T qc[9], const T wk[9],
                                                const T y[9], const int pos[3], const int N[3], const T a[3][3],

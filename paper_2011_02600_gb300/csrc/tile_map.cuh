@@ -1,7 +1,8 @@
-// Tile geometry of the tiled stage kernel (kernels_tiled.cu): tile size and halo, the node
+// Tile geometry of the tiled stage kernel (kernels_tiled.cuh): tile size and halo, the node
 // range each tile owns along q and r, the launch order of the tiles, the per-thread rows of D-
-// and D+ along q, the closure-row sums along s, and the length of the chunks along s.  Device code of the kernel; without nvcc the same source compiles as
-// host C++, so that the index arithmetic can be checked for any grid size on a CPU.
+// and D+ along q, the closure-row sums along s, and the length of the chunks along s.  Device
+// code of the kernel; without nvcc the same source compiles as host C++, so that the index
+// arithmetic can be checked for any grid size on a CPU.
 #pragma once
 
 #include "common.cuh"
