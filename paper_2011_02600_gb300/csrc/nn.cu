@@ -849,7 +849,7 @@ int sbp_nn_bias_grad(const void* dZ, float* db, int32_t M, int64_t N, void* stre
   const cudaStream_t st = (cudaStream_t)stream;
   const int wide = N % 8 == 0 && aligned16(dZ);
   if (N <= 2048)
-    bias_grad_kernel<32><<<(M + 7) / 8, 256, 0, st>>>((const __nv_bfloat16*)dZ, db, M, N, wide);
+    bias_grad_kernel<32><<<M / 8 + (M % 8 != 0), 256, 0, st>>>((const __nv_bfloat16*)dZ, db, M, N, wide);
   else
     bias_grad_kernel<256><<<M, 256, 0, st>>>((const __nv_bfloat16*)dZ, db, M, N, wide);
   return nn_status(cudaGetLastError());
