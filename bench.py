@@ -336,9 +336,10 @@ def run_adjoint(args, local):
     peak = peaks["hbm_gbs"] if peaks else 6800.0
     topo = s.map_path() == "topography"
     adj_bytes = ADJ_BYTES_PER_NODE_STAGE_TOPO if topo else ADJ_BYTES_PER_NODE_STAGE
-    # the forward stage kernel's bytes, averaged over the five stages (stage 0 reads no RK register)
-    stage_bytes = ((BYTES_PER_NODE_STAGE0_TOPO + 4 * BYTES_PER_NODE_STAGE_TOPO) / 5 if topo else
-                   (BYTES_PER_NODE_STAGE0 + 4 * BYTES_PER_NODE_STAGE) / 5)
+    # the forward stage kernel's bytes, averaged over a step's 14 launches (five in the forward run, five
+    # in the recomputation, four for the stage inputs; stage 0 reads no RK register)
+    stage_bytes = ((3 * BYTES_PER_NODE_STAGE0_TOPO + 11 * BYTES_PER_NODE_STAGE_TOPO) / 14 if topo else
+                   (3 * BYTES_PER_NODE_STAGE0 + 11 * BYTES_PER_NODE_STAGE) / 14)
     achieved = adj_bytes * nodes / (adj_avg / 1e3) / 1e9
     value = nodes * 5 * nsteps / ((t_fwd + t_grad) / 1e3) / 1e6
     line = {
