@@ -348,7 +348,7 @@ int sbp_adjoint_step(SbpGrid* grid, double dt, const void* u_stages, void* ubar,
  * group of states (5 groups of 9 B fields, grid layout) and receives U_1 .. U_4 in the
  * others, at the grid's time (sbp_set_time; the source's stage times).  Uses the
  * Runge-Kutta register; the bound state, time and step counter stay as they are.
- * u_stages: 256-byte aligned, not a bound buffer.
+ * u_stages: 256-byte aligned; its bytes overlap no bound buffer (SBP_ERR_ARG otherwise).
  * Errors: UNSUPPORTED on slab grids and with interface faces. */
 int sbp_stage_inputs(SbpGrid* grid, double dt, void* u_stages, void* stream);
 

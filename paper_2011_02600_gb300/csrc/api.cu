@@ -423,6 +423,11 @@ int stage_inputs_impl(SbpGrid* g, double dt, T* u, cudaStream_t st) {
   return SBP_OK;
 }
 
+// Whether [p, p + np) and [q, q + nq) share a byte.
+bool overlap(const void* p, size_t np, const void* q, size_t nq) {
+  return (uintptr_t)p < (uintptr_t)q + nq && (uintptr_t)q < (uintptr_t)p + np;
+}
+
 int check_ready(const SbpGrid* g) {
   if (!g) return fail(SBP_ERR_ARG, "null grid");
   if (!g->bound) return fail(SBP_ERR_STATE, "buffers not bound (sbp_bind)");
@@ -785,8 +790,12 @@ int sbp_stage_inputs(SbpGrid* g, double dt, void* u_stages, void* stream) {
   if (int rc = check_ready(g)) return rc;
   if (!g->material) return fail(SBP_ERR_STATE, "material not set (sbp_set_material)");
   if (!u_stages || (uintptr_t)u_stages % 256) return fail(SBP_ERR_ARG, "stage buffer null or not 256-byte aligned");
-  if (u_stages == g->q[0] || u_stages == g->q[1] || u_stages == g->dq)
-    return fail(SBP_ERR_ARG, "the stage buffer aliases a bound buffer");
+  const size_t field = (size_t)g->dims.fs * g->elem, state = 9 * field * g->nb;
+  const std::pair<const void*, size_t> held[5] = {
+      {g->q[0], state}, {g->q[1], state}, {g->dq, state}, {g->met, 9 * field}, {g->mat, 3 * field}};
+  for (const auto& h : held)
+    if (overlap(u_stages, 5 * state, h.first, h.second))
+      return fail(SBP_ERR_ARG, "the stage buffer overlaps a bound buffer");
   if (!(dt > 0) || !isfinite(dt)) return fail(SBP_ERR_ARG, "dt must be positive and finite");
   if (has_interface(g) || g->slab.ns_global > 0)
     return fail(SBP_ERR_UNSUPPORTED, "stage inputs need a block of their own (no interface faces, no slab)");

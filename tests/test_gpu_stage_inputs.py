@@ -62,3 +62,22 @@ def test_gradient_leaves_the_solver_after_the_first_step():
     p._reset()
     p.s.step(1, c["dt"])
     assert np.array_equal(left.cpu().numpy(), p.s.qbuf[p.s.current].cpu().numpy())
+
+
+@pytest.mark.parametrize("batch", [1, 2])
+def test_stage_inputs_refuse_a_buffer_that_overlaps_a_bound_one(batch):
+    """Refused before any launch: a buffer that starts inside a bound one, at its first and its last
+    aligned address, or that runs into one.  The bytes behind the addresses are not touched."""
+    from paper_2011_02600_gb300 import _lib as L
+    c = _misfit_case(nsteps=1)
+    p, _ = _batched_problem(c, _three_sources()[:batch])
+    _set(p, c["mat"])
+    s = p.s
+    field = s.fs * s.met.element_size()
+    state = 9 * batch * field
+    for buf, size in ((s.qbuf[0], state), (s.qbuf[1], state), (s.dq, state), (s.met, 9 * field), (s.mat, 3 * field)):
+        base = buf.data_ptr()
+        for at in (base, base + 256, base + size - 256, base - 5 * state + 256):
+            with pytest.raises(L.SbpError) as e:
+                L.sbp_stage_inputs(s.h, c["dt"], at, None)
+            assert e.value.code == 1 and "overlap" in str(e.value)
