@@ -31,3 +31,28 @@ def test_register_of_the_first_stage_is_dt_times_the_rate(precision, nodes, path
     s.rk_stage(0, dt)
     want = torch.tensor(dt, dtype=s.dtype, device=rate.device) * rate
     assert torch.equal(s.view(s.dq, 9), want)
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+@pytest.mark.parametrize("nodes,extent", [((36, 22, 40), (20000.0, 13000.0, 15000.0)),
+                                          ((47, 31, 20), (7000.0, 9500.0, 5000.0))])
+def test_strain_rates_on_topography_maps_round_once_per_product(precision, nodes, extent):
+    """Order 2 with velocities linear in the node index and lambda = 0: the derivative times N - 1 is a
+    whole number, so that sigma_xx and sigma_yy away from the faces are mu/J a (N - 1) dv with one rounding
+    per product of the kernel's (and one for a_r = c a_q,x), bit for bit."""
+    from paper_2011_02600_gb300.workload_setup import build_solver
+    cfg = dataclasses.replace(config_by_name("hill129_o6"), nodes=nodes, extent=extent, order=2)
+    s, _ = build_solver(cfg, precision=precision, keep_metrics=True)
+    assert s.map_path() == "topography"
+    s.view(s.mat, 3)[1].zero_()                              # lambda / J
+    jq, mu2 = s.view(s.met, 9)[0], 2 * s.view(s.mat, 3)[2]
+    jm = s.view(s.jmet, 10)
+    c = (jm[5, 0, 0, 0] / jm[1, 0, 0, 0]).to(s.dtype)
+    inner = (slice(2, -2),) * 3
+    for f in (1, 3, 5, 7, 11, 25):
+        Q = torch.zeros(9, *reversed(nodes), dtype=s.dtype)
+        Q[0] = f * torch.arange(nodes[0], dtype=s.dtype)
+        Q[1] = f * torch.arange(nodes[1], dtype=s.dtype)[:, None]
+        rate = s.rhs(Q)
+        for row, a, n in ((3, jq, nodes[0]), (4, c * jq, nodes[1])):
+            assert torch.equal(rate[row][inner], (mu2 * (a * (f * (n - 1.0))))[inner]), (f, row)
