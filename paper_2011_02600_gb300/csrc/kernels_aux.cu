@@ -61,9 +61,10 @@ cudaError_t launch_topography_check(const double* jmet, const Dims& d, double c,
 }
 
 // ---------------------------------------------------------------------------
-// Solver coefficients: met = a (cast), mat = (1/(rho J), lambda/J, mu/J).  One FP64 division per node
-// (1/J = rho (1/(rho J))) and the sign tests on the bits: with three divisions and five FP64
-// comparisons the pass was bound by the FP64 pipe; 257 x 257 x 129: 602 -> 338 us.
+// Solver coefficients: met = a (cast), mat = (1/(rho J), lambda/J, mu/J), kept for a whole run: in FP64
+// the quotients themselves, one rounding each; in FP32 products with 1/J, whose FP64 roundings are 2^-29
+// of the one to FP32.  Sign tests on the bits: with three divisions and five FP64 comparisons the pass
+// was bound by the FP64 pipe; 257 x 257 x 129, FP32: 602 -> 410 us.
 template <typename T>
 __global__ void __launch_bounds__(256) material_kernel(const double* __restrict__ jmet, const double* __restrict__ rlm,
                                                        T* __restrict__ met, T* __restrict__ mat, Dims d,
@@ -77,10 +78,15 @@ __global__ void __launch_bounds__(256) material_kernel(const double* __restrict_
 #pragma unroll
   for (int c = 0; c < 9; ++c) met[c * d.fs + n0] = (T)jmet[(1 + c) * d.fs + n0];
   const double rho = rlm[n0], lam = rlm[d.fs + n0], mu = rlm[2 * d.fs + n0];
-  const double irJ = 1.0 / (rho * J), iJ = irJ * rho;
-  mat[n0] = (T)irJ;
-  mat[d.fs + n0] = (T)(lam * iJ);
-  mat[2 * d.fs + n0] = (T)(mu * iJ);
+  mat[n0] = (T)(1.0 / (rho * J));
+  if (sizeof(T) == 8) {
+    mat[d.fs + n0] = (T)(lam / J);
+    mat[2 * d.fs + n0] = (T)(mu / J);
+  } else {
+    const double iJ = 1.0 / J;
+    mat[d.fs + n0] = (T)(lam * iJ);
+    mat[2 * d.fs + n0] = (T)(mu * iJ);
+  }
   auto positive = [](double x) { return positive_bits(__double_as_longlong(x)); };
   if (!positive(rho) || !positive(mu) || !positive(lam + 2.0 * mu)) atomicOr(status, 4u);
   if (!positive(J)) atomicOr(status, 2u);
