@@ -25,8 +25,9 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
     add_strain(a, u, sb);
     return;
   }
-  T n[3];
-  const T an = face_normal(a, n);
+  T ian;
+  const T an = face_length(a, ian);
+  const T n[3] = {quotient(a[0], an, ian), quotient(a[1], an, ian), quotient(a[2], an, ian)};
   const Impedances<T> Z = impedances(irhoJ, lamJ, muJ);
   const T f = an * inv_h0;
   const T fsg = side == 0 ? f : -f;
@@ -36,10 +37,10 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
   flux(n, ys, w);  // traction of y_sigma on the face
   const T un = yv[0] * n[0] + yv[1] * n[1] + yv[2] * n[2];
   const T wn = w[0] * n[0] + w[1] * n[1] + w[2] * n[2];
-  const T an_ = -f * un + fsg * wn * Z.iZp;
+  const T an_ = -f * un + quotient(fsg * wn, Z.Zp, Z.iZp);
   T at[3];
 #pragma unroll
-  for (int c = 0; c < 3; ++c) at[c] = -f * (yv[c] - un * n[c]) + fsg * (w[c] - wn * n[c]) * Z.iZs;
+  for (int c = 0; c < 3; ++c) at[c] = -f * (yv[c] - un * n[c]) + quotient(fsg * (w[c] - wn * n[c]), Z.Zs, Z.iZs);
 #pragma unroll
   for (int c = 0; c < 3; ++c) vb[c] += cv * (Z.Zp * an_ * n[c] + Z.Zs * at[c]);
   const T beta[3] = {cT * (an_ * n[0] + at[0]), cT * (an_ * n[1] + at[1]), cT * (an_ * n[2] + at[2])};
@@ -49,10 +50,11 @@ __device__ __forceinline__ void add_penalty_transpose(int side, int kind, T gamm
 // d/dZp and d/dZs of y . SAT(U) for the general penalty (U = (v, sigma) at the node).
 template <typename T>
 __device__ __forceinline__ void penalty_impedance_derivs(int side, T gamma, T inv_h0, const T v[3], const T s[6],
-                                                         const T yv[3], const T ys[6], const T a[3], T iZp, T iZs,
-                                                         T& dZp, T& dZs) {
-  T n[3];
-  const T an = face_normal(a, n);
+                                                         const T yv[3], const T ys[6], const T a[3],
+                                                         const Impedances<T>& Z, T& dZp, T& dZs) {
+  T ian;
+  const T an = face_length(a, ian);
+  const T n[3] = {quotient(a[0], an, ian), quotient(a[1], an, ian), quotient(a[2], an, ian)};
   const T f = an * inv_h0;
   const T fsg = side == 0 ? f : -f;
   const T cv = T(0.5) * (T(1) - gamma);
@@ -70,8 +72,8 @@ __device__ __forceinline__ void penalty_impedance_derivs(int side, T gamma, T in
     vtut += (v[c] - vn * n[c]) * (yv[c] - un * n[c]);
     Ttwt += (Tr[c] - Tn * n[c]) * (w[c] - wn * n[c]);
   }
-  dZp = -f * cv * vn * un - fsg * cT * Tn * wn * (iZp * iZp);
-  dZs = -f * cv * vtut - fsg * cT * Ttwt * (iZs * iZs);
+  dZp = -f * cv * vn * un - quotient(fsg * cT * Tn * wn, Z.Zp * Z.Zp, Z.iZp * Z.iZp);
+  dZs = -f * cv * vtut - quotient(fsg * cT * Ttwt, Z.Zs * Z.Zs, Z.iZs * Z.iZs);
 }
 
 // Face terms of L^T at one node: for each face the node lies on, (B H^-1)_xi applied to
@@ -138,8 +140,7 @@ __device__ __forceinline__ void gradient_terms(const T rv[3], const T e[6], cons
       if ((side == 0 && !lo) || (side == 1 && !hi)) continue;
       if (bc_kind[2 * xi + side] != 1) continue;
       T dZp, dZs;
-      penalty_impedance_derivs<T>(side, bc_gamma[2 * xi + side], inv_h0[xi], qc, qc + 3, y, y + 3, a[xi], Z.iZp, Z.iZs,
-                                  dZp, dZs);
+      penalty_impedance_derivs<T>(side, bc_gamma[2 * xi + side], inv_h0[xi], qc, qc + 3, y, y + 3, a[xi], Z, dZp, dZs);
       d_rho += (dZp * Z.Zp + dZs * Z.Zs) * i2r;
       d_lam += dZp * rT * T(0.5) * Z.iZp;
       d_mu += dZp * rT * Z.iZp + dZs * rT * T(0.5) * Z.iZs;

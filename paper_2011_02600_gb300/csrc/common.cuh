@@ -212,8 +212,8 @@ __device__ __forceinline__ void add_strain(const T a[3], const T dv[3], T e[6]) 
   e[5] += a[2] * dv[1] + a[1] * dv[2];
 }
 
-// 1 / sqrt(x): one instruction sequence on the device (at most 1 ulp off in FP64, 2 in FP32) in place
-// of a square root and a division.
+// 1 / sqrt(x), a few ulp off on the device (the CUDA documentation: 1 in FP64, 2 in FP32): the first
+// value of the corrections below.
 __host__ __device__ __forceinline__ double inv_sqrt(double x) {
 #ifdef __CUDA_ARCH__
   return rsqrt(x);
@@ -229,32 +229,55 @@ __host__ __device__ __forceinline__ float inv_sqrt(float x) {
 #endif
 }
 
-// |a| and n = a / |a|.
+// Newton steps with the residual formed by a fused multiply-add (Markstein 1990): from a value a few ulp
+// off to one within 1 ulp, the last addition's rounding and next to nothing.
+// 1/d from about 1/d.
 template <typename T>
-__device__ __forceinline__ T face_normal(const T a[3], T n[3]) {
+__device__ __forceinline__ T corrected_reciprocal(T d, T id) {
+  return fma(fma(-d, id, T(1)), id, id);
+}
+// x/d from id, about 1/d.
+template <typename T>
+__device__ __forceinline__ T quotient(T x, T d, T id) {
+  const T q = x * id;
+  return fma(fma(-q, d, x), id, q);
+}
+
+// |a| and ia = 1/|a|.
+template <typename T>
+__device__ __forceinline__ T face_length(const T a[3], T& ia) {
   const T a2 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2];
-  const T ian = inv_sqrt(a2);
-  n[0] = a[0] * ian;
-  n[1] = a[1] * ian;
-  n[2] = a[2] * ian;
-  return a2 * ian;
+  const T y = inv_sqrt(a2), x = a2 * y;
+  const T an = fma(fma(-x, x, a2), T(0.5) * y, x);
+  ia = corrected_reciprocal(an, y);
+  return an;
 }
 
 // Impedances Z_p = sqrt((lambda + 2 mu) rho), Z_s = sqrt(mu rho) and their reciprocals from the
-// stored 1/(rho J), lambda/J, mu/J: Z = sqrt(c) / sqrt(r) with c the modulus over J and r = 1/(rho J),
-// each root on its own, so that no product of the two leaves the range of FP32.
-// With a square root or a division at a time a face node's penalty was as much FP64 work as its
-// stencils, and every warp of a tile at a face waits for it: per stage, 129 x 129 x 97 order 6 1.37
-// -> 1.33 ms in FP64, 125 -> 122 us in FP32; 33^3 order 4 FP64 104 -> 101 us.
+// stored 1/(rho J), lambda/J, mu/J: the root of r Z^2 = c with c the modulus over J and r = 1/(rho J).
 template <typename T>
 struct Impedances {
   T Zp, Zs, iZp, iZs;
 };
+// First by p = 1/sqrt(r c), the product of two reciprocal roots (no product of r and c leaves the range of
+// FP32), then one Newton step.  Its residual c - (r z) z carries the rounding of r z: the error bounds of
+// sqrt(c / r), 1.5 (Z_s) and 2 (Z_p) units of roundoff, which the uncorrected products exceed.  Every warp of
+// a tile at a face waits for this; uncorrected, corrected, and with square roots and divisions: 97^3 order 4
+// FP32, 64 members, 2 steps 27.3, 27.5, 28.6 ms; a 16-step gradient of 8 sources on 129 x 129 x 97 289, 291,
+// 311 ms; that grid at order 6 in FP64, 2 steps 12.4, 12.7, 12.8 ms; 33^3 FP64, 10 steps 4.05, 4.24, 4.15 ms.
+template <typename T>
+__device__ __forceinline__ void impedance(T c, T r, T ir, T& Z, T& iZ) {
+  const T p = inv_sqrt(c) * ir, z = c * p;
+  Z = fma(fma(-(r * z), z, c), T(0.5) * p, z);
+  iZ = corrected_reciprocal(Z, r * p);
+}
 template <typename T>
 __device__ __forceinline__ Impedances<T> impedances(T irhoJ, T lamJ, T muJ) {
-  const T cp = lamJ + T(2) * muJ;
-  const T ip = inv_sqrt(cp), is = inv_sqrt(muJ), ir = inv_sqrt(irhoJ), r = irhoJ * ir;
-  return Impedances<T>{cp * ip * ir, muJ * is * ir, r * ip, r * is};
+  const T ir = inv_sqrt(irhoJ);
+  Impedances<T> I;
+  impedance(fma(T(2), muJ, lamJ), irhoJ, ir, I.Zp, I.iZp);
+  impedance(muJ, irhoJ, ir, I.Zs, I.iZs);
+  return I;
 }
 
 // Penalty of one face at one face node, added to the velocity rows rv and the
@@ -280,8 +303,9 @@ __device__ __forceinline__ void add_penalty(int side, int kind, T gamma, T inv_h
     rv[2] += sg * Fa[2];
     return;
   }
-  T n[3], Tr[3];
-  const T an = face_normal(a, n);
+  T ian, Tr[3];
+  const T an = face_length(a, ian);
+  const T n[3] = {a[0] * ian, a[1] * ian, a[2] * ian};
   flux(n, s, Tr);
   const Impedances<T> Z = impedances(irhoJ, lamJ, muJ);
   const T vn = v[0] * n[0] + v[1] * n[1] + v[2] * n[2];
@@ -322,8 +346,9 @@ __device__ __forceinline__ void add_penalty(int side, int kind, T gamma, T inv_h
 template <typename T>
 __device__ __forceinline__ void add_interface_penalty(int side, T inv_h0, const T v[3], const T s[6], const T a[3],
                                                       T irhoJ, T lamJ, T muJ, const T o[8], T rv[3], T e[6]) {
-  T n[3], Tr[3];
-  const T an = face_normal(a, n);
+  T ian, Tr[3];
+  const T an = face_length(a, ian);
+  const T n[3] = {a[0] * ian, a[1] * ian, a[2] * ian};
   flux(n, s, Tr);
   const Impedances<T> Zi = impedances(irhoJ, lamJ, muJ);
   const T Zp = Zi.Zp, Zs = Zi.Zs;

@@ -293,9 +293,9 @@ __global__ void interface_trace_kernel(const T* __restrict__ q, const T* __restr
   const long long fs = d.fs;
   const T* qb = q + (long long)b * bstride;
   const T a[3] = {met[(3 * xi) * fs + n0], met[(3 * xi + 1) * fs + n0], met[(3 * xi + 2) * fs + n0]};
-  const T ian = T(1) / sqrt(a[0] * a[0] + a[1] * a[1] + a[2] * a[2]);
+  T ian, sg[6], Tr[3];
+  face_length(a, ian);
   const T n[3] = {a[0] * ian, a[1] * ian, a[2] * ian};
-  T sg[6], Tr[3];
 #pragma unroll
   for (int c = 0; c < 6; ++c) sg[c] = qb[(3 + c) * fs + n0];
   flux(n, sg, Tr);
@@ -305,8 +305,9 @@ __global__ void interface_trace_kernel(const T* __restrict__ q, const T* __restr
   for (int c = 0; c < 3; ++c) out[c * nf] = qb[c * fs + n0];
 #pragma unroll
   for (int c = 0; c < 3; ++c) out[(3 + c) * nf] = Tr[c];
-  out[6 * nf] = sqrt((lamJ + T(2) * muJ) / irhoJ);
-  out[7 * nf] = sqrt(muJ / irhoJ);
+  const Impedances<T> Z = impedances(irhoJ, lamJ, muJ);  // as in the penalty they enter
+  out[6 * nf] = Z.Zp;
+  out[7 * nf] = Z.Zs;
 }
 
 template <typename T>
