@@ -446,9 +446,11 @@ __global__ void relu_bwd_kernel(const float* __restrict__ dA, const __nv_bfloat1
     dZ[e] = __float2bfloat16(__bfloat162float(A[e]) > 0.f ? dA[e] : 0.f);
 }
 
-// db[m] = sum_n dZ[m][n], fixed order: TPR threads per row (a warp for short rows, else a block), a
-// thread's values 8 at a time where `wide` (rows 16-byte aligned).  1152 x 32768 (75 MB): 21 -> 14 us;
-// 4096 x 32: 7.2 -> 3.0 us (a block per row had 32 of its 256 threads at work).
+// db[m] = sum_n dZ[m][n], fixed order: TPR threads per row (a warp for short rows, else a block), eight
+// sums a thread, added pairwise with the other threads', so that a value passes through at most
+// ceil(N / 256) + 8 additions, as with a thread per value and block; its values 8 at a time where `wide`
+// (rows 16-byte aligned).  A call against a thread per value and block: 1152 x 32768 (75 MB, not in L2) 31
+// -> 21 us, 4096 x 32 10 -> 6 us.
 template <int TPR>
 __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __restrict__ dZ, float* __restrict__ db,
                                                         int M, long long N, int wide) {
@@ -456,16 +458,21 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
   const int m = blockIdx.x * (256 / TPR) + threadIdx.x / TPR, lane = threadIdx.x % TPR;
   if (TPR < 256 && m >= M) return;  // whole warps
   const __nv_bfloat16* row = dZ + (size_t)m * N;
-  float s = 0.f;
+  float p[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   if (wide) {
     for (long long n = 8 * lane; n < N; n += 8 * TPR) {
       const Bf8 x = *reinterpret_cast<const Bf8*>(row + n);
 #pragma unroll
-      for (int e = 0; e < 8; ++e) s += __bfloat162float(x.v[e]);
+      for (int e = 0; e < 8; ++e) p[e] += __bfloat162float(x.v[e]);
     }
   } else {
-    for (long long n = lane; n < N; n += TPR) s += __bfloat162float(row[n]);
+    for (long long n = lane; n < N; n += 8 * TPR) {
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if (n + e * TPR < N) p[e] += __bfloat162float(row[n + e * TPR]);
+    }
   }
+  float s = ((p[0] + p[4]) + (p[2] + p[6])) + ((p[1] + p[5]) + (p[3] + p[7]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   if (TPR == 32) {
@@ -474,12 +481,7 @@ __global__ void __launch_bounds__(256) bias_grad_kernel(const __nv_bfloat16* __r
   }
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
   __syncthreads();
-  if (threadIdx.x == 0) {
-    float v = 0.f;
-#pragma unroll
-    for (int w = 0; w < TPR / 32; ++w) v += red[w];
-    db[m] = v;
-  }
+  if (threadIdx.x == 0) db[m] = ((red[0] + red[4]) + (red[2] + red[6])) + ((red[1] + red[5]) + (red[3] + red[7]));
 }
 
 // mean squared error over n values: per-block FP64 partial sums of (y - t)^2 and dY = 2 (y - t) / n (BF16)
