@@ -208,6 +208,11 @@ int sbp_step_n(SbpGrid* grid, int32_t n, double dt, void* stream);
  * 1 = the general one-thread-per-node kernel over every node.  Both compute
  * the same scheme; path 1 exists to cross-check the tiled kernel. */
 int sbp_set_kernel_path(SbpGrid* grid, int32_t path);
+/* Planes along s that a block of the tiled kernel marches through: 0 (default) =
+ * chosen from the grid's size; a positive count is taken as given (at most the
+ * grid's planes).  The results do not depend on it: it exists to check that, as
+ * the choice for a small grid is one or two planes. */
+int sbp_set_chunk(SbpGrid* grid, int32_t planes);
 
 /* Per-kernel timing: when enabled, each stage-kernel launch is bracketed by
  * CUDA events recorded on the launching stream.  sbp_kernel_times waits for

@@ -31,7 +31,7 @@ EXPORTED = ("sbp_min_nodes", "sbp_create_grid", "sbp_destroy", "sbp_layout", "sb
             "sbp_nn_set_gemm_path", "sbp_nn_status", "sbp_set_slab", "sbp_interface_trace", "sbp_set_interface",
             "sbp_probe_fp64_rate", "sbp_set_map_path", "sbp_map_path", "sbp_adjoint_step",
             "sbp_nn_fourier_features", "sbp_nn_upsample_im2col", "sbp_nn_conv_relu_backward", "sbp_nn_adam_multi",
-            "sbp_stage_inputs")
+            "sbp_stage_inputs", "sbp_set_chunk")
 
 
 class SbpError(RuntimeError):
@@ -78,6 +78,7 @@ def lib(path=None):
         "sbp_rk_stage": [P, i32, dbl, P],
         "sbp_step_n": [P, i32, dbl, P],
         "sbp_set_kernel_path": [P, i32],
+        "sbp_set_chunk": [P, i32],
         "sbp_set_map_path": [P, i32],
         "sbp_map_path": [P, ctypes.POINTER(i32)],
         "sbp_current": [P, ctypes.POINTER(i32)],
@@ -205,6 +206,10 @@ def sbp_step_n(h, n, dt, stream):
 
 def sbp_set_kernel_path(h, path):
     _check(lib().sbp_set_kernel_path(h, path))
+
+
+def sbp_set_chunk(h, planes):
+    _check(lib().sbp_set_chunk(h, planes))
 
 
 def sbp_set_map_path(h, path):

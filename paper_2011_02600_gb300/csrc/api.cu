@@ -167,6 +167,7 @@ struct SbpGrid {
   bool topo = false;
   double ar_ratio = 0.0;  // a_r,y / a_q,x
   int map_path = SBP_MAP_AUTO;
+  int chunk = 0;  // sbp_set_chunk
   // tensor maps of the tiled stage kernel, per state buffer (q0, q1)
   bool tma_ok[2] = {false, false};
   sbp::TmaSet tma[2];
@@ -247,6 +248,7 @@ sbp::StageArgs<T> make_args(const SbpGrid* g, const void* q, void* qout, int mod
   A.status = g->status;
   A.sclose = (T*)g->sclose;
   A.sc_bstride = sclose_elems(g);
+  A.chunk = g->chunk;
   A.slab = g->slab;
   A.map = uses_topography(g) ? 1 : 0;
   A.ar_ratio = (T)g->ar_ratio;
@@ -838,6 +840,13 @@ int sbp_set_kernel_path(SbpGrid* g, int32_t path) {
   if (!g) return fail(SBP_ERR_ARG, "null grid");
   if (path != 0 && path != 1) return fail(SBP_ERR_ARG, "kernel path must be 0 or 1");
   g->use_tiled = path == 0;
+  return SBP_OK;
+}
+
+int sbp_set_chunk(SbpGrid* g, int32_t planes) {
+  if (!g) return fail(SBP_ERR_ARG, "null grid");
+  if (planes < 0) return fail(SBP_ERR_ARG, "negative number of planes");
+  g->chunk = planes;
   return SBP_OK;
 }
 

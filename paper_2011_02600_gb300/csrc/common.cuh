@@ -77,6 +77,7 @@ struct StageArgs {
   long long bstride;  // elements between consecutive states (9 fields)
   T* sclose;          // tiled kernel scratch: s-closure sums, 2 b 6 planes per state
   long long sc_bstride;  // elements between consecutive states' scratch
+  int chunk;             // planes a block of the tiled kernel marches through; 0: s_chunk's choice
   // adjoint passes of the tiled kernel (q is then yhat = H^-1 P~ Wb_k, or U_k)
   const T* ubar_next;   // Ub_{k+1} (null: zero)
   T* ubar_out;          // Ub_k, or L^T w (mode kModeRhs)

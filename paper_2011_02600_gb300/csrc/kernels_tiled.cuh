@@ -693,9 +693,10 @@ cudaError_t launch_tiled_order(const StageArgs<T>& A, const TmaSet& tm, cudaStre
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     sms = 152;  // GB300
   const long long tiles = (long long)((ni + TX - 1) / TX) * ((nj + TY - 1) / TY) * A.nb;
-  const int chunk = sizeof(T) == 4
-                        ? s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(), NVQ<O>() * 0.6, OpCoef<O>::b, 6)
-                        : s_chunk(tiles, nk, A.nb, (long long)sms * tiled_min_blocks<T>(), NVQ<O>() / 6.0, OpCoef<O>::b, 1);
+  const long long slots = (long long)sms * tiled_min_blocks<T>();
+  const int chunk = A.chunk > 0     ? min(A.chunk, nk)
+                    : sizeof(T) == 4 ? s_chunk(tiles, nk, A.nb, slots, NVQ<O>() * 0.6, OpCoef<O>::b, 6)
+                                     : s_chunk(tiles, nk, A.nb, slots, NVQ<O>() / 6.0, OpCoef<O>::b, 1);
   dim3 grid((ni + TX - 1) / TX, (nj + TY - 1) / TY, ((nk + chunk - 1) / chunk) * A.nb);
   if (grid.z > 65535 || grid.y > 65535) return cudaErrorInvalidConfiguration;
   dim3 block(TX, TY);
