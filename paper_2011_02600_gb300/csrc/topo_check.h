@@ -46,15 +46,6 @@ __host__ __device__ inline long long abs_bits(double x) {
 #endif
   return b & 0x7fffffffffffffffLL;
 }
-__host__ __device__ inline double from_bits(long long b) {
-#ifdef __CUDA_ARCH__
-  return __longlong_as_double(b);
-#else
-  double x;
-  memcpy(&x, &b, sizeof x);
-  return x;
-#endif
-}
 __host__ __device__ inline bool topography_within(const double* jmet, long long fs, double c, double tol,
                                                   long long n0) {
   const double aqx = jmet[1 * fs + n0], ary = jmet[5 * fs + n0];
