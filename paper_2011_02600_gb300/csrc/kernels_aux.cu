@@ -113,6 +113,7 @@ template cudaError_t launch_material<double>(const double*, const double*, doubl
 constexpr int kEnergyBlocks = 1184;  // 152 SMs x 8
 constexpr int kEnergyThreads = 256;
 int energy_blocks() { return kEnergyBlocks; }
+constexpr int kEnergyPairRow = 224;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -120,12 +121,14 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// One warp per (r, s) row of nodes (q contiguous), two neighbouring nodes per lane and load where
-// `pairs` (FP32, 8-byte aligned rows); rows strided over the grid.  The row's weights along q are 1
-// but for the closures' nodes, and the spacing is taken out of the sum, so that a node costs the
-// FP64 pipe a conversion and an addition; with a weight per node the pipe bound the pass.  385 x 385
-// x 193 FP32 (1.37 GB): 345 -> 259 us.  A slab of a decomposed block sums its own planes only, with the
-// block's weights along s.
+// One warp per (r, s) row of nodes (q contiguous); rows strided over the grid.  The spacings and the
+// row's weights are taken out of the sum, so that a node costs the FP64 pipe a conversion and a
+// multiply-add; with a weight per node the pipe bound the pass.  `pairs` (FP32, 8-byte aligned rows of
+// at least kEnergyPairRow nodes): two neighbouring nodes per lane and load, and no weight inside.  Calls
+// at order 6, a weight per node / pairs / single nodes: 385 x 385 x 193 (1.37 GB) 371 / 285 / 298 us, 257 x 257 x
+// 129 148 / 124 / 124, 160 x 200 x 200 113 / 111 / 99, 60 x 300 x 300 126 / 114 / 102, 30 x 300 x 300 98 / 113 /
+// 86: pairs leave up to three quarters of the lanes of a short row idle, and the line lies where they stop losing.  A
+// slab of a decomposed block sums its own planes only, with the block's weights along s.
 template <typename T, int O>
 __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(const T* __restrict__ q, const T* __restrict__ mat,
                                                                 Dims d, SlabS sl, int pairs,
@@ -176,7 +179,9 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(const T* __restr
         T f[12];
 #pragma unroll
         for (int c = 0; c < 12; ++c) f[c] = c < 9 ? q[c * fs + n0] : mat[(c - 9) * fs + n0];
-        add(i, f);
+        const T dens = energy_density<T>(f, f + 3, f[9], f[10], f[11]);
+        bad |= !isfinite(dens);
+        racc += norm_weight_t<double, O>(i, d.nq) * (double)dens;
       }
     }
     acc += wjk * racc;
@@ -210,7 +215,7 @@ __global__ void sum_partials_kernel(const double* __restrict__ partial, int n, d
 template <typename T>
 cudaError_t launch_energy(const T* q, const T* mat, const Dims& d, int order, double* partial, int nblocks,
                           double* out, unsigned* status, cudaStream_t st, SlabS sl) {
-  const int pairs = ((uintptr_t)q | (uintptr_t)mat) % 8 == 0 && d.ldq % 2 == 0 && d.plane % 2 == 0 && d.fs % 2 == 0;
+  const int pairs = d.nq >= kEnergyPairRow && ((uintptr_t)q | (uintptr_t)mat) % 8 == 0 && d.ldq % 2 == 0 && d.plane % 2 == 0 && d.fs % 2 == 0;
   switch (order) {
     case 2: energy_kernel<T, 2><<<nblocks, kEnergyThreads, 0, st>>>(q, mat, d, sl, pairs, partial, status); break;
     case 4: energy_kernel<T, 4><<<nblocks, kEnergyThreads, 0, st>>>(q, mat, d, sl, pairs, partial, status); break;
