@@ -155,6 +155,7 @@ int sbp_bind(SbpGrid* grid, void* q0, void* q1, void* dq, void* met, void* mat);
  * D_c = (D+ + D-)/2 of the upwind pair of the grid's order, also for the
  * traditional operators) into jmet (10 FP64 fields: J, then
  * the 9 metrics; device, caller-owned).  Flags SBP_STATUS_BAD_MESH where J <= 0.
+ * Only nodes are read and written: the padding of either buffer may hold anything.
  * On a slab grid every inner end needs at least the reach of that D_c in ghost
  * planes (for the traditional operators one more than sbp_set_slab asks):
  * SBP_ERR_ARG otherwise. */
@@ -162,7 +163,8 @@ int sbp_metrics(SbpGrid* grid, const double* xyz, double* jmet, void* stream);
 
 /* Fill the bound met (a[xi][eta] cast to the solver precision) and mat
  * (1/(rho J), lambda/J, mu/J) from jmet (as produced by sbp_metrics) and rlm
- * (3 FP64 fields rho, lambda, mu; device).  Flags SBP_STATUS_BAD_MATERIAL where
+ * (3 FP64 fields rho, lambda, mu; device); only their nodes are read, not the
+ * padding.  Flags SBP_STATUS_BAD_MATERIAL where
  * rho <= 0, mu <= 0 or lambda + 2 mu <= 0.  Also finds whether the metrics are
  * those of a topography map x = L_x q, y = L_y r, z = z(q, r, s) (the configs'
  * layered and topographic grids): then a_q = (a_q,x, 0, 0) and a_r =

@@ -32,3 +32,24 @@ def test_coefficients(precision, name, nodes):
     want = torch.stack([1.0 / (rho * J), lam / J, mu / J]).to(s.dtype)
     assert torch.isfinite(want).all()
     assert torch.equal(s.view(s.mat, 3), want)
+
+
+def test_padding_is_not_read():
+    """Only the nodes of the coordinates, metrics and moduli count: NaN between the rows changes nothing."""
+    from paper_2011_02600_gb300 import ElasticSolver
+    from paper_2011_02600_gb300 import _lib as L
+    from workloads.media import make_medium
+    nodes = (37, 21, 18)
+    X = np.stack(node_coordinates(make_map("gaussian_hill", (20000.0, 19000.0, 15000.0)), nodes))
+    mat = np.stack(make_medium("smooth_gradient", Lz=15000.0)(*X))
+    a, b = (ElasticSolver(nodes, 4, 32, [("free",)] * 6) for _ in range(2))
+    a.setup(torch.from_numpy(X), torch.from_numpy(mat), keep_metrics=True)
+    xyz, jmet, rlm = (torch.full((n * b.fs,), float("nan"), dtype=torch.float64, device="cuda") for n in (3, 10, 3))
+    b.view(xyz, 3).copy_(torch.from_numpy(X))
+    b.view(rlm, 3).copy_(torch.from_numpy(mat))
+    st = torch.cuda.current_stream().cuda_stream
+    L.sbp_metrics(b.h, xyz, jmet, st)
+    L.sbp_set_material(b.h, jmet, rlm, st)
+    assert b.status() == 0 and b.map_path() == a.map_path() == "topography"
+    assert torch.equal(b.view(jmet, 10), a.view(a.jmet, 10))
+    assert torch.equal(b.view(b.met, 9), a.view(a.met, 9)) and torch.equal(b.view(b.mat, 3), a.view(a.mat, 3))
