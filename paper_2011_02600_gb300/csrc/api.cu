@@ -415,7 +415,8 @@ int stage_impl(SbpGrid* g, int k, double dt, cudaStream_t st) {
 // The stage inputs U_1 .. U_4 of a step from U_0, back to back in u: four stages (the fifth would only
 // give the next step's state, which the adjoint has), each writing where the next one and the adjoint
 // read.  Bound by the stages themselves (0.59 ms each, 8 members of 129 x 129 x 97, FP32); with five stages
-// through the bound buffers and five copies (0.155 ms each) a 16-step gradient took 311.8 ms, so 288.6.  The tensor
+// through the bound buffers and five copies (0.155 ms each) a 16-step gradient took 311.8 ms, so 288.6
+// (290.5 with the corrected penalties of common.cuh).  The tensor
 // maps of u are encoded per call, a few microseconds beside a stage: nothing is kept by u's address.
 template <typename T>
 int stage_inputs_impl(SbpGrid* g, double dt, T* u, cudaStream_t st) {

@@ -484,7 +484,8 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
       ar_at(st, HX + ty, tx, c_r, a);
       strain_r<MAP>(a, dv, e);
     } else if (active) {
-      // closure row of a node within b of an r face (whole warps: the row is uniform)
+      // closure row of a node within b of an r face (a row per warp: uniform in it; the nodes of a packed
+      // tile's warps lie on several rows)
       const bool lo = j < BC;
       const int row = lo ? j : d.nr - 1 - j;
       T sf[3] = {T(0), T(0), T(0)}, sv[3] = {T(0), T(0), T(0)};
@@ -665,7 +666,8 @@ __global__ void __launch_bounds__(TX* TY, tiled_min_blocks<T>())
         double g[3];
         gradient_terms(rv, e, qc, pre, y, pos, N, a, irhoJ, lamJ, muJ, rj[0], rj[1], A.bc_kind, A.bc_gamma,
                        A.inv_h0, (double)A.dt, g);
-        // one writer per node and launch: a reduction that needs no read-back
+        // the members of a batch add to the same node, in no fixed order: atomic, and a reduction that
+        // needs no read-back
 #pragma unroll
         for (int c = 0; c < 3; ++c) atomicAdd(A.grad + (c * fs + (long long)k * d.plane) + at, g[c]);
       }

@@ -676,12 +676,12 @@ int nn_bad(const char* msg) {
 // GEMM path (sbp_nn_set_gemm_path): 0 automatic, 1 mma.sync kernels only, 2 tcgen05 whenever possible.
 int g_gemm_path = 0;
 
-// SM count of the current device (152 on GB300, also the value taken if the query fails).
 bool aligned16(const void* p) { return (uintptr_t)p % 16 == 0; }
 // Rows of B * T columns that a thread can take eight of at a time: one sample's, 16-byte aligned, and
 // few enough for 32-bit indices and a grid row each.
 bool by_eight(long long B, long long T, long long rows) { return T % 8 == 0 && B * T < (1LL << 31) - 2048 && rows <= 65535; }
 
+// SM count of the current device (152 on GB300, also the value taken if the query fails).
 int device_sms() {
   int dev = 0, n = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||

@@ -184,9 +184,13 @@ __device__ __forceinline__ void s_closure_sums(const T* __restrict__ q, const T*
 // for the loads, a sixth in FP64, where the pipe counts).  The last chunk also forms the closure
 // sums at s = 1 (`extra` planes' time), and the one before it does when the last holds fewer than the
 // b closure planes.  Large grids take few long chunks, small ones are cut until the rounds even out.
+// The form is that of a plan in rounds; its weights (0.6 and a sixth of the queues, 6 and 1 planes for the
+// closure sums whatever their width, one and the same cost for every tile) were fitted to the stage times of
+// four grids, not derived: the length chosen is within some 12 % of the best one.  86 x 187 x 133 order 4 FP32: 14
+// planes, 590 us a step; 34 planes, one full round, 552.
 // Per stage, against at most 96 planes and no fewer than 16: 33^3 order 4 FP64 (20 blocks on 152 SMs)
-// 481 -> 79 us; 129 x 129 x 97 order 6 FP64 (170 blocks) 2.35 -> 1.18 ms, FP32 (255 blocks on 304
-// slots) 137 -> 112 us; 257 x 241 x 161 curvilinear FP32 629 -> 514 us, other gains of this kernel
+// 481 -> 85 us; 129 x 129 x 97 order 6 FP64 (170 blocks) 2.35 -> 1.27 ms, FP32 (255 blocks on 304
+// slots) 137 -> 113 us; 257 x 241 x 161 curvilinear FP32 629 -> 522 us, other gains of this kernel
 // included; 769 x 769 x 257 takes 3 chunks (6 cost 1 %, 16 cost 8 %).
 inline int s_chunk(long long tiles, int nk, int nb, long long slots, double warm, int b, int extra) {
   int best = nk;
